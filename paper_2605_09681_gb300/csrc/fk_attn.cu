@@ -7,10 +7,10 @@
 //                      maps over the view arenas) into two-stage rings, 128-byte swizzle;
 //                      key tile 0 on its own barrier, then V_j together with K_{j+1} on one
 //                      barrier per stage pair (one wait and one release per key tile);
-//   warp 9 (one lane)  tcgen05.mma, per key tile j: P_0 V_j, S_0(j+1), P_1 V_j, S_1(j+1)
+//   warp 9             tcgen05.mma, per key tile j: P_0 V_j, S_0(j+1), P_1 V_j, S_1(j+1)
 //                      (S_t = Q_t K^T into TMEM, O_t += P_t V with P_t read from TMEM);
-//                      completion via tcgen05.commit; the barriers of the next group are
-//                      tested without blocking while the tensor pipe still runs this one;
+//                      completion via tcgen05.commit; the warp stays converged and an elected
+//                      lane issues (see elect_one);
 //   warps 0-3 / 4-7    softmax of query tile 0 / 1 (ping-pong: one warpgroup's softmax
 //                      overlaps the other tile's MMAs): thread r owns row r = TMEM lane r,
 //                      reads S with tcgen05.ld, online softmax in the log2 domain with a
@@ -112,16 +112,6 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
-// Non-blocking test of the phase of parity `parity` (acquire when it has completed).
-__device__ __forceinline__ bool mbar_peek(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok) : "r"(su32(b)), "r"(parity) : "memory");
-  return ok != 0;
-}
-
 // Bounded wait for the phase of parity `parity`.  Returns false when the CTA is
 // aborting or the limit expired (which starts the abort).  Inlined: a call would save and
 // restore the caller's live registers on every wait, even when the phase is complete.
@@ -186,6 +176,15 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int b_mn) {
 // 7 and 10), A K-major, B K-major (b_mn = 0) or MN-major (b_mn = 1).
 __host__ __device__ constexpr uint32_t idesc_e4m3(int M, int N, int b_mn = 0) {
   return (1u << 4) | ((uint32_t)b_mn << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// One lane of the (converged) warp, the same one each time.  tcgen05.mma and commit behind this
+// predicate take their operands from uniform registers; behind `lane == 0` the compiler does not
+// know that one lane is left, and an MMA cost 80-100 cycles of issue whatever its size.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e != 0;
 }
 
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
@@ -457,83 +456,76 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // one thread complete in issue order, so when S_t(j+1) is reported complete, PV_t(j)
     // is complete too: the softmax of tile j+1 may rescale O_t without a further wait, and
     // S_t(j+1) overwriting P_t(j) (same columns) happens after PV_t(j) has read it.
-    if (lane == 0) {
-      constexpr uint32_t kIdQK = kFp8 ? idesc_e4m3(kAttnBM, kAttnBN) : idesc_bf16(kAttnBM, kAttnBN, 0);
-      constexpr uint32_t kIdPV = kFp8PV ? idesc_e4m3(kAttnBM, D, 1) : idesc_bf16(kAttnBM, D, 1);
-      const uint32_t aQ = su32(sQ), aK = su32(sK), aV = su32(sV);
-      auto qk = [&](int j, int t) {
-        const int st = j & 1;
-        if constexpr (kFp8) {
-          // 128 codes per row = one swizzle atom: four K = 32 steps of 32 bytes
+    constexpr uint32_t kIdQK = kFp8 ? idesc_e4m3(kAttnBM, kAttnBN) : idesc_bf16(kAttnBM, kAttnBN, 0);
+    constexpr uint32_t kIdPV = kFp8PV ? idesc_e4m3(kAttnBM, D, 1) : idesc_bf16(kAttnBM, D, 1);
+    const uint64_t dQ = sdesc(su32(sQ), 16, 1024), dK = sdesc(su32(sK), 16, 1024);
+    const uint64_t dV = sdesc(su32(sV), 16384, 1024);
+    auto qk = [&](int j, int t) {
+      const uint64_t da = dQ + (uint32_t)(t * (Lay::kQ >> 4)), db = dK + (uint32_t)((j & 1) * (Lay::kK >> 4));
+      const uint32_t d = tmem + (uint32_t)(t * kAttnBN);
+      if constexpr (kFp8) {
+        // 128 codes per row = one swizzle atom: four K = 32 steps of 32 bytes
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t da = sdesc(aQ + t * Lay::kQ + kk * 32, 16, 1024);
-            const uint64_t db = sdesc(aK + st * Lay::kK + kk * 32, 16, 1024);
-            umma_f8(tmem + (uint32_t)(t * kAttnBN), da, db, kIdQK, kk > 0 ? 1u : 0u);
-          }
-        } else {
+        for (int kk = 0; kk < 4; ++kk) umma_f8(d, da + kk * 2, db + kk * 2, kIdQK, kk > 0 ? 1u : 0u);
+      } else {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t da = sdesc(aQ + t * Lay::kQ + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
-            const uint64_t db = sdesc(aK + st * Lay::kK + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
-            umma(tmem + (uint32_t)(t * kAttnBN), da, db, kIdQK, kk > 0 ? 1u : 0u);
-          }
+        for (int kk = 0; kk < D / 16; ++kk) {
+          const uint32_t off = (uint32_t)((kk >> 2) * 1024 + (kk & 3) * 2);
+          umma(d, da + off, db + off, kIdQK, kk > 0 ? 1u : 0u);
         }
-        umma_commit(&bar->s_full[t]);
-      };
-      auto pv = [&](int j, int t) {
-        const int st = j & 1;
-        if constexpr (kFp8PV) {
-          // 32 keys per step: P columns 8 kk .. 8 kk + 7 (four codes each); V rows 32 kk .. +31,
-          // MN-major (d contiguous, 128 bytes per key row), 8-row groups 1024 bytes apart
+      }
+      umma_commit(&bar->s_full[t]);
+    };
+    auto pv = [&](int j, int t) {
+      const uint64_t db = dV + (uint32_t)((j & 1) * (Lay::kKV >> 4));
+      const uint32_t d = tmem + kColO + (uint32_t)(t * D), p = tmem + (uint32_t)(t * kAttnBN);
+      if constexpr (kFp8PV) {
+        // 32 keys per step: P columns 8 kk .. 8 kk + 7 (four codes each); V rows 32 kk .. +31,
+        // MN-major (d contiguous, 128 bytes per key row), 8-row groups 1024 bytes apart
 #pragma unroll
-          for (int kk = 0; kk < kAttnBN / 32; ++kk) {
-            const uint64_t db = sdesc(aV + st * Lay::kKV + kk * 4096, 16384, 1024);
-            umma_ts_f8(tmem + kColO + (uint32_t)(t * D), tmem + (uint32_t)(t * kAttnBN + kk * 8), db,
-                       kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
-          }
-        } else {
+        for (int kk = 0; kk < kAttnBN / 32; ++kk)
+          umma_ts_f8(d, p + kk * 8, db + kk * 256, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
+      } else {
 #pragma unroll
-          for (int kk = 0; kk < kAttnBN / 16; ++kk) {
-            const uint64_t db = sdesc(aV + st * Lay::kKV + kk * 2048, 16384, 1024);
-            umma_ts(tmem + kColO + (uint32_t)(t * D), tmem + (uint32_t)(t * kAttnBN + kk * 8), db,
-                    kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
-          }
-        }
-      };
-      bool ok = wait_phase(kFp8 ? &bar->q8_ready : &bar->q_full, 0, bar, a.status) &&
-                wait_phase(&bar->k0_full, 0, bar, a.status);
-      if (ok) {
-        tc_fence_after();
+        for (int kk = 0; kk < kAttnBN / 16; ++kk)
+          umma_ts(d, p + kk * 8, db + kk * 128, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
+      }
+    };
+    // every lane waits, one issues: the warp stays converged
+    auto wait = [&](uint64_t* b, uint32_t parity) { return warp_wait(b, parity, bar, a.status); };
+    bool ok = wait(kFp8 ? &bar->q8_ready : &bar->q_full, 0) && wait(&bar->k0_full, 0);
+    if (ok) {
+      tc_fence_after();
+      if (elect_one()) {
         qk(0, 0);
         qk(0, 1);
         umma_commit(&bar->k0_empty);
       }
-      // barriers found complete by a test made while the pipe was busy with the group just issued
-      // need no wait afterwards (each wait costs ~100 cycles where the pipe would drain)
-      bool vk_ready = false;
-      for (int j = 0; j < nt && ok; ++j) {
-        const int bb = j & 1;
-        const bool more = j + 1 < nt;
-        // V_j and K_{j+1} (one barrier) before P_0(j): neither depends on the softmax, and
-        // PV0(j), S0(j+1) then go to the tensor pipe back to back once P_0(j) is in TMEM
-        if (!(vk_ready || wait_phase(&bar->vk_full[bb], (j >> 1) & 1, bar, a.status)) ||
-            !wait_phase(&bar->p_full[0], j & 1, bar, a.status)) { ok = false; break; }
-        tc_fence_after();
-        pv(j, 0);
-        const bool p1_ready = mbar_peek(&bar->p_full[1], j & 1);
-        if (more) qk(j + 1, 0);
-        if (!(p1_ready || wait_phase(&bar->p_full[1], j & 1, bar, a.status))) { ok = false; break; }
-        tc_fence_after();
-        pv(j, 1);
-        vk_ready = more && mbar_peek(&bar->vk_full[(j + 1) & 1], ((j + 1) >> 1) & 1);
-        if (more) qk(j + 1, 1);
-        umma_commit(&bar->vk_empty[bb]);             // V_j and K_{j+1} consumed
-      }
-      if (ok) umma_commit(&bar->o_done);
-      umma_commit(&bar->fin);                       // completes once every MMA above is done
-      wait_phase(&bar->fin, 0, bar, a.status, false);
     }
+    for (int j = 0; j < nt && ok; ++j) {
+      const int bb = j & 1;
+      const bool more = j + 1 < nt;
+      // V_j and K_{j+1} (one barrier) before P_0(j): neither depends on the softmax, and
+      // PV0(j), S0(j+1) then go to the tensor pipe back to back once P_0(j) is in TMEM
+      if (!wait(&bar->vk_full[bb], (j >> 1) & 1) || !wait(&bar->p_full[0], j & 1)) { ok = false; break; }
+      tc_fence_after();
+      if (elect_one()) {
+        pv(j, 0);
+        if (more) qk(j + 1, 0);
+      }
+      if (!wait(&bar->p_full[1], j & 1)) { ok = false; break; }
+      tc_fence_after();
+      if (elect_one()) {
+        pv(j, 1);
+        if (more) qk(j + 1, 1);
+        umma_commit(&bar->vk_empty[bb]);           // V_j and K_{j+1} consumed
+      }
+    }
+    if (elect_one()) {
+      if (ok) umma_commit(&bar->o_done);
+      umma_commit(&bar->fin);                     // completes once every MMA above is done
+    }
+    wait_phase(&bar->fin, 0, bar, a.status, false);
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ softmax warpgroups
@@ -963,27 +955,27 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
     __syncwarp();
   } else if (warp == kWarpProfMma) {
-    if (lane == 0) {
-      constexpr uint32_t kIdQK = idesc_bf16(kAttnBM, kAttnBN, 0);
-      const uint32_t aQ = su32(sQ), aK = su32(sK);
-      bool ok = wait_phase(&bar->q_full, 0, bar, a.status);
-      for (int j = 0; j < nt && ok; ++j) {
-        const int st = j & 1, u = j >> 1;
-        if (!wait_phase(&bar->k_full[st], u & 1, bar, a.status) ||
-            (j >= 2 && !wait_phase(&bar->p_full[st], (u - 1) & 1, bar, a.status))) { ok = false; break; }
-        tc_fence_after();
+    constexpr uint32_t kIdQK = idesc_bf16(kAttnBM, kAttnBN, 0);
+    const uint64_t dQ = sdesc(su32(sQ), 16, 1024), dK = sdesc(su32(sK), 16, 1024);
+    bool ok = warp_wait(&bar->q_full, 0, bar, a.status);
+    for (int j = 0; j < nt && ok; ++j) {
+      const int st = j & 1, u = j >> 1;
+      if (!warp_wait(&bar->k_full[st], u & 1, bar, a.status) ||
+          (j >= 2 && !warp_wait(&bar->p_full[st], (u - 1) & 1, bar, a.status))) { ok = false; break; }
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t db = dK + (uint32_t)(st * (Lay::kK >> 4));
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t da = sdesc(aQ + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
-          const uint64_t db = sdesc(aK + st * Lay::kK + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
-          umma(tmem + (uint32_t)(st * kAttnBN), da, db, kIdQK, kk > 0 ? 1u : 0u);
+          const uint32_t off = (uint32_t)((kk >> 2) * 1024 + (kk & 3) * 2);
+          umma(tmem + (uint32_t)(st * kAttnBN), dQ + off, db + off, kIdQK, kk > 0 ? 1u : 0u);
         }
         umma_commit(&bar->s_full[st]);
         umma_commit(&bar->k_empty[st]);
       }
-      umma_commit(&bar->fin);                       // completes once every MMA above is done
-      wait_phase(&bar->fin, 0, bar, a.status, false);
     }
+    if (elect_one()) umma_commit(&bar->fin);      // completes once every MMA above is done
+    wait_phase(&bar->fin, 0, bar, a.status, false);
     __syncwarp();
   } else {
     const int wq = warp;
