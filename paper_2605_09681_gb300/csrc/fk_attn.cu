@@ -7,19 +7,28 @@
 //                      maps over the view arenas) into two-stage rings, 128-byte swizzle;
 //                      key tile 0 on its own barrier, then V_j together with K_{j+1} on one
 //                      barrier per stage pair (one wait and one release per key tile);
-//   warp 9             tcgen05.mma, per key tile j: P_0 V_j, S_0(j+1), P_1 V_j, S_1(j+1)
+//   warp 9             tcgen05.mma, per key tile j and query tile t: P_t V_j of keys 0-95, of
+//                      keys 96-127 (each once its P is in TMEM), then S_t(j+1)
 //                      (S_t = Q_t K^T into TMEM, O_t += P_t V with P_t read from TMEM);
 //                      completion via tcgen05.commit; the warp stays converged and an elected
 //                      lane issues (see elect_one);
 //   warps 0-3 / 4-7    softmax of query tile 0 / 1 (ping-pong: one warpgroup's softmax
 //                      overlaps the other tile's MMAs): thread r owns row r = TMEM lane r,
 //                      reads S with tcgen05.ld, online softmax in the log2 domain with a
-//                      lazily rescaled running max, writes P as bf16 pairs over S's first
-//                      64 columns with tcgen05.st, and finally normalises O and stores it.
-//                      After the first key tile a 64-key half computes P with the running
-//                      max at once; its sum (at most 2^8) or the packed maximum of its P
-//                      shows that no numerator exceeds the rescale bound, else the half is
-//                      redone with a max pass.
+//                      lazily raised running max, writes P as bf16 pairs over S columns already
+//                      read with tcgen05.st, and finally normalises O and stores it.  A key tile
+//                      goes to the MMA warp in two parts, keys 0-95 and 96-127, so that P V of the
+//                      first runs while the second is computed.  After the first key tile a part's
+//                      P is computed with the running max at once; its sum (at most 2^8) shows
+//                      that no numerator exceeds that bound, else the part is done again with
+//                      a max pass that raises the running max and rescales O and the row sum.
+//                      What bounds it (clock64 timeline of one CTA, 12 heads x 25480 keys, D =
+//                      128): one key tile takes 2500 cycles for 2048 cycles of MMA; a tile's
+//                      softmax takes 1090 of them and its P waits ~500 for the tensor pipe.  One
+//                      hand-over per tile, a vote and a store wait per 64 columns and S kept for
+//                      both took 1230; a denoising step then ran 321 us (now 304), a step under
+//                      FP8 Q K^T 326 us (now 290), a 1080P step 6.22 ms (now 5.61).  96 + 32:
+//                      P V of the first part (384 cycles) covers the second's arithmetic (~190).
 // TMEM columns: S0 0-127, S1 128-255, O0 256.., O1 256+D.. (512 allocated).
 // FP8_QK variant (D = 128): the K tiles hold E4M3 codes (one 128-byte swizzle atom per row,
 // from the view arena's E4M3 copy); the bf16 Q tiles are loaded as usual and each softmax
@@ -44,7 +53,7 @@ namespace fk {
 namespace {
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s per wait
-constexpr float kRescaleThreshold = 8.0f;          // log2 units: rescale O when max grows > 2^8
+constexpr float kRescaleThreshold = 1.0f;          // log2 units: a part that exceeds the bound raises m
 // FP8 P V: P is stored as e4m3 of 2^6 exp2(s c - m), m an integer running reference (the
 // running max rounded up) that lags the row max by at most 2 (rescale threshold), so P stays
 // within 2^8 < 448; reference changes rescale O and l by exact powers of two
@@ -61,6 +70,7 @@ struct AttnBarriers {
   uint64_t k0_full, k0_empty;       // attention: key tile 0 (stage 0)
   uint64_t vk_full[2], vk_empty[2]; // attention, b = j mod 2: V_j (V stage b) with K_{j+1} (K stage 1-b)
   uint64_t s_full[2], p_full[2];
+  uint64_t pa_full[2], pva_done[2];  // attention: P of a tile's first 96 keys written / multiplied
   uint64_t o_done, fin;
   uint64_t q8_ready;            // FP8_QK: the 256 softmax threads have written the E4M3 Q rows
   uint32_t tmem_base;
@@ -266,14 +276,10 @@ __device__ __forceinline__ void umma_commit(uint64_t* b) {
         "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]),  \
         "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]) : "memory")
 
-#define FK_TMEM_LD16(taddr, v)                                                              \
-  asm volatile(                                                                             \
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"  \
-      "%13,%14,%15}, [%16];"                                                                \
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),  \
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),           \
-        "=r"(v[13]), "=r"(v[14]), "=r"(v[15])                                               \
-      : "r"(taddr))
+#define FK_TMEM_ST8(taddr, v)                                                               \
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"     \
+               :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),        \
+               "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory")
 
 #define FK_TMEM_ST16(taddr, v)                                                              \
   asm volatile(                                                                             \
@@ -312,19 +318,60 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return d;
 }
 
-// four e4m3 codes (one TMEM column of P, lowest key in the low byte) times alpha, re-rounded
-__device__ __forceinline__ uint32_t scale_e4m3x4(uint32_t w, float alpha) {
-  uint32_t lo, hi;
-  asm("{\n .reg .b16 a, b;\n mov.b32 {a, b}, %2;\n cvt.rn.f16x2.e4m3x2 %0, a;\n"
-      " cvt.rn.f16x2.e4m3x2 %1, b;\n}" : "=r"(lo), "=r"(hi) : "r"(w));
-  const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&lo));
-  const float2 f1 = __half22float2(*reinterpret_cast<const __half2*>(&hi));
-  return e4m3x2(f0.x * alpha, f0.y * alpha) | (e4m3x2(f1.x * alpha, f1.y * alpha) << 16);
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// tcgen05.wait::ld that also names the registers of the loads it completes, so that no use of
+// them can be scheduled before it
+#define FK_TMEM_WAIT_LD32(v)                                                                \
+  asm volatile("tcgen05.wait::ld.sync.aligned;"                                             \
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),    \
+                 "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]),  \
+                 "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]),           \
+                 "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]),           \
+                 "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]),           \
+                 "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])            \
+               :: "memory")
+
+// 32 logits -> numerators exp2(s * sc + nm): their sums in four chains, and P words (bf16 pairs, or
+// four E4M3 codes; `ov` then collects the bits of the overflow test).  The sums and roundings of a
+// pair come kSkew pairs after its exponentials, so that they do not wait for them.
+constexpr int kSkew = 4;
+template <bool kE4m3>
+__device__ __forceinline__ void exp_chunk(const uint32_t* s, float2 sc2, float2 nm2, float2* ah,
+                                          uint32_t* pk, uint32_t& ov) {
+  float2 e[16];
+#pragma unroll
+  for (int q = 0; q < 16 + kSkew; ++q) {
+    if (q < 16) {
+      const float2 x = ffma2(make_float2(__uint_as_float(s[2 * q]), __uint_as_float(s[2 * q + 1])), sc2, nm2);
+      e[q] = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+    }
+    if (q >= kSkew) {
+      const int p = q - kSkew;
+      ah[p & 3] = fadd2(ah[p & 3], e[p]);
+      if constexpr (kE4m3) {
+        if (p & 1) {
+          pk[p >> 1] = e4m3x2(e[p - 1].x, e[p - 1].y) | (e4m3x2(e[p].x, e[p].y) << 16);
+          ov |= pk[p >> 1] + 0x07070707u;
+        }
+      } else {
+        pk[p] = pack_bf16(e[p].x, e[p].y);
+      }
+    }
+  }
+}
+
+// Whether a numerator of these columns may exceed 2^8 in any lane (warp-uniform).  bf16: no more
+// than their sum does.  E4M3: exactly when a code is above 0x78; codes are non-negative and at
+// most 0x7E, so adding 7 to each byte sets its top bit then, without carries between bytes.
+template <bool kE4m3>
+__device__ __forceinline__ bool exceeds(const float2* ah, uint32_t ov) {
+  if constexpr (kE4m3) return __any_sync(0xffffffffu, (ov & 0x80808080u) != 0);
+  const float2 hs2 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
+  return __any_sync(0xffffffffu, hs2.x + hs2.y > 256.0f);
 }
 
 // kSplit: a launch with key splits (kv_splits > 1); the unsplit instantiation carries none of
@@ -379,6 +426,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       mbar_init(&bar->vk_empty[i], 1);
       mbar_init(&bar->s_full[i], 1);
       mbar_init(&bar->p_full[i], 4);
+      mbar_init(&bar->pa_full[i], 4);
+      mbar_init(&bar->pva_done[i], 1);
     }
     mbar_init(&bar->o_done, 1);
     mbar_init(&bar->fin, 1);
@@ -476,18 +525,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       }
       umma_commit(&bar->s_full[t]);
     };
-    auto pv = [&](int j, int t) {
+    // PV of a tile's keys 32 c0 .. 32 c1 - 1
+    auto pv = [&](int j, int t, int c0, int c1) {
       const uint64_t db = dV + (uint32_t)((j & 1) * (Lay::kKV >> 4));
       const uint32_t d = tmem + kColO + (uint32_t)(t * D), p = tmem + (uint32_t)(t * kAttnBN);
       if constexpr (kFp8PV) {
         // 32 keys per step: P columns 8 kk .. 8 kk + 7 (four codes each); V rows 32 kk .. +31,
         // MN-major (d contiguous, 128 bytes per key row), 8-row groups 1024 bytes apart
 #pragma unroll
-        for (int kk = 0; kk < kAttnBN / 32; ++kk)
+        for (int kk = c0; kk < c1; ++kk)
           umma_ts_f8(d, p + kk * 8, db + kk * 256, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
       } else {
 #pragma unroll
-        for (int kk = 0; kk < kAttnBN / 16; ++kk)
+        for (int kk = 2 * c0; kk < 2 * c1; ++kk)
           umma_ts(d, p + kk * 8, db + kk * 128, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
       }
     };
@@ -507,18 +557,22 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       const bool more = j + 1 < nt;
       // V_j and K_{j+1} (one barrier) before P_0(j): neither depends on the softmax, and
       // PV0(j), S0(j+1) then go to the tensor pipe back to back once P_0(j) is in TMEM
-      if (!wait(&bar->vk_full[bb], (j >> 1) & 1) || !wait(&bar->p_full[0], j & 1)) { ok = false; break; }
-      tc_fence_after();
-      if (elect_one()) {
-        pv(j, 0);
-        if (more) qk(j + 1, 0);
-      }
-      if (!wait(&bar->p_full[1], j & 1)) { ok = false; break; }
-      tc_fence_after();
-      if (elect_one()) {
-        pv(j, 1);
-        if (more) qk(j + 1, 1);
-        umma_commit(&bar->vk_empty[bb]);           // V_j and K_{j+1} consumed
+      if (!wait(&bar->vk_full[bb], (j >> 1) & 1)) { ok = false; break; }
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (!wait(&bar->pa_full[t], j & 1)) { ok = false; break; }
+        tc_fence_after();
+        if (elect_one()) {
+          pv(j, t, 0, 3);
+          umma_commit(&bar->pva_done[t]);
+        }
+        if (!wait(&bar->p_full[t], j & 1)) { ok = false; break; }
+        tc_fence_after();
+        if (elect_one()) {
+          pv(j, t, 3, 4);
+          if (more) qk(j + 1, t);
+          if (t == 1) umma_commit(&bar->vk_empty[bb]);   // V_j and K_{j+1} consumed
+        }
       }
     }
     if (elect_one()) {
@@ -568,118 +622,36 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       }
       mbar_arrive(&bar->q8_ready);
     }
+    const float2 sc2 = make_float2(sl2, sl2);
     float m = -INFINITY, l = 0.0f;
     for (int j = 0; j < nt && ok; ++j) {
       if (!warp_wait(&bar->s_full[t], j & 1, bar, a.status)) { ok = false; break; }
       tc_fence_after();
       const int valid = nk - j * kAttnBN;           // keys of this tile (< 128 only in the last)
-      const bool full = valid >= kAttnBN;           // uniform over the CTA
-      const float2 sc2 = make_float2(sl2, sl2);
-      float2 acc[4];
+      // A tile goes in two parts, keys 0-95 and 96-127, each handed to the MMA warp as soon as
+      // its P is in TMEM.  P = exp2(S*c - m) is written over S columns already read (bf16 pairs:
+      // P columns 16c..16c+15 come from S columns 32c..32c+31; FP8 P V: e4m3 codes of
+      // 2^6 exp2(S*c - m), four per column, P columns 8c..8c+7): the A operand of PV.  On full
+      // tiles after the first, P is computed with the running max m straight away, the next
+      // 32 columns' load in flight; a part whose numerators all stay within 2^8 is stored, else it
+      // is done again by general_part.
+      // general_part: chunks [c0, c1) with a max pass, and m raised when it grows by more than kThr
+      // (FP8 P V: m is the running max rounded up to an integer).  O_t holds PV of every key before
+      // part c0: with part 0 PV_t(j-1) is complete (see MMA order), with part 1 the keys of part 0
+      // once pva_done says so.
+      auto general_part = [&](int c0, int c1) -> bool {
+        float mx = -INFINITY;
+#pragma unroll 1
+        for (int c = c0; c < c1; ++c) {
+          uint32_t sv[32];
+          FK_TMEM_LD32(tS + c * 32, sv);
+          FK_TMEM_WAIT_LD32(sv);
+          float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.0f, 0.0f);
-      float alpha_tile = 1.0f;
-      bool rescaled = false;
-      // One pass per 64-column half: the half's maximum (eight independent chains), a lazy
-      // update of the running max m (only when it grows by more than 2^8), then
-      // P = exp2(S*c - m) as bf16 pairs written over the S columns already read (P columns
-      // 32h..32h+31 come from S columns 64h..64h+63): the A operand of PV.  FP8 P V: m is the
-      // running max rounded up to an integer, updated when it grows by more than 2, and P the
-      // e4m3 codes of 2^6 exp2(S*c - m), four per column (P columns 16h..16h+15).  If the second
-      // half raises m, the first half's stored P is rescaled in place.
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t sv[64];
-        FK_TMEM_LD64(tS + half * 64, sv);
-        tmem_wait_ld();
-        if constexpr (!kFp8PV) {
-          // Full tile after the first (every row has a finite running max m): P = exp2(S*c - m)
-          // straight away; m has to move only if some P exceeds 2^8 (an element more than 8
-          // above m), which the packed bf16 maximum of the half's P shows.  Otherwise the
-          // half is done without a separate max pass; if it does, the path below redoes it.
-          if (full && j > 0) {
-            uint32_t pk[32];
-            float2 ah[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
-            const float2 nm2 = make_float2(-m, -m);
-#pragma unroll
-            for (int q = 0; q < 32; ++q) {
-              const float2 x = ffma2(make_float2(__uint_as_float(sv[2 * q]), __uint_as_float(sv[2 * q + 1])),
-                                     sc2, nm2);
-              float2 e;
-              e.x = fast_exp2(x.x);
-              e.y = fast_exp2(x.y);
-              ah[q & 3] = fadd2(ah[q & 3], e);
-              pk[q] = pack_bf16(e.x, e.y);
-            }
-            // the half's sum bounds each of its numerators: only a sum above 2^8 needs the max
-            const float2 hs2 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
-            bool over = false;
-            if (__any_sync(0xffffffffu, hs2.x + hs2.y > 256.0f)) {
-              __nv_bfloat162 pm[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) pm[i] = *reinterpret_cast<const __nv_bfloat162*>(&pk[i]);
-#pragma unroll
-              for (int q = 4; q < 32; ++q)
-                pm[q & 3] = __hmax2(pm[q & 3], *reinterpret_cast<const __nv_bfloat162*>(&pk[q]));
-              const __nv_bfloat162 p2 = __hmax2(__hmax2(pm[0], pm[1]), __hmax2(pm[2], pm[3]));
-              over = fmaxf(__low2float(p2), __high2float(p2)) > 256.0f;
-            }
-            if (!__any_sync(0xffffffffu, over)) {                          // warp-uniform
-#pragma unroll
-              for (int i = 0; i < 4; ++i) acc[i] = fadd2(acc[i], ah[i]);
-              FK_TMEM_ST32(tS + half * 32, pk);
-              continue;
-            }
-          }
-        } else {
-          // FP8 P V, the same idea with the integer reference: a numerator above 2^8 (y more than
-          // 2 above m) shows as an e4m3 code above 0x78; codes are non-negative and at most 0x7E,
-          // so adding 7 to each byte sets its top bit exactly then, without carries between bytes
-          if (full && j > 0) {
-            uint32_t pk[16], ov = 0;
-            float2 ah[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
-            const float2 nm2 = make_float2(kPShift - m, kPShift - m);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              const float2 x0 = ffma2(make_float2(__uint_as_float(sv[4 * q]), __uint_as_float(sv[4 * q + 1])),
-                                      sc2, nm2);
-              const float2 x1 = ffma2(make_float2(__uint_as_float(sv[4 * q + 2]), __uint_as_float(sv[4 * q + 3])),
-                                      sc2, nm2);
-              float2 e0, e1;
-              e0.x = fast_exp2(x0.x);
-              e0.y = fast_exp2(x0.y);
-              e1.x = fast_exp2(x1.x);
-              e1.y = fast_exp2(x1.y);
-              ah[(2 * q) & 3] = fadd2(ah[(2 * q) & 3], e0);
-              ah[(2 * q + 1) & 3] = fadd2(ah[(2 * q + 1) & 3], e1);
-              pk[q] = e4m3x2(e0.x, e0.y) | (e4m3x2(e1.x, e1.y) << 16);
-              ov |= pk[q] + 0x07070707u;
-            }
-            if (!__any_sync(0xffffffffu, (ov & 0x80808080u) != 0)) {   // warp-uniform
-#pragma unroll
-              for (int i = 0; i < 4; ++i) acc[i] = fadd2(acc[i], ah[i]);
-              FK_TMEM_ST16(tS + half * 16, pk);
-              continue;
-            }
-          }
+          for (int i = 0; i < 32; ++i)
+            if (c * 32 + i < valid) mxa[i & 3] = fmaxf(mxa[i & 3], __uint_as_float(sv[i]));
+          mx = fmaxf(mx, fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])));
         }
-        float mxa[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mxa[i] = -INFINITY;
-        if (full) {
-#pragma unroll
-          for (int c = 0; c < 64; ++c) mxa[c & 7] = fmaxf(mxa[c & 7], __uint_as_float(sv[c]));
-        } else {
-#pragma unroll
-          for (int c = 0; c < 64; ++c)
-            if (half * 64 + c < valid) mxa[c & 7] = fmaxf(mxa[c & 7], __uint_as_float(sv[c]));
-        }
-        const float mx = fmaxf(fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])),
-                               fmaxf(fmaxf(mxa[4], mxa[5]), fmaxf(mxa[6], mxa[7])));
         const float m_new = fmaxf(m, kFp8PV ? ceilf(mx * sl2) : mx * sl2);
         if (__any_sync(0xffffffffu, m_new > m + kThr)) {               // warp-uniform
           float alpha;                               // 0 when m = -inf
@@ -690,105 +662,102 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             alpha = fast_exp2(m - m_new);
           }
           l *= alpha;
+          m = m_new;
+          if (c0 > 0) {
+            if (!warp_wait(&bar->pva_done[t], j & 1, bar, a.status)) return false;
+            tc_fence_after();
+          }
+          if (j > 0 || c0 > 0) {
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+              uint32_t o[32];
+              FK_TMEM_LD32(tO + c * 32, o);
+              FK_TMEM_WAIT_LD32(o);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) acc[i] = make_float2(acc[i].x * alpha, acc[i].y * alpha);
-          if (half == 1) {                           // rare: first half of P was stored with the old m
-            if constexpr (kFp8PV) {
-              uint32_t p0[16];
-              tmem_wait_st();
-              FK_TMEM_LD16(tS, p0);
-              tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 16; ++e) p0[e] = scale_e4m3x4(p0[e], alpha);
-              FK_TMEM_ST16(tS, p0);
-            } else {
-              uint32_t p0[32];
-              tmem_wait_st();
-              FK_TMEM_LD32(tS, p0);
-              tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&p0[e]);
-                p0[e] = pack_bf16(__low2float(b) * alpha, __high2float(b) * alpha);
-              }
-              FK_TMEM_ST32(tS, p0);
+              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              FK_TMEM_ST32(tO + c * 32, o);
             }
           }
-          alpha_tile *= alpha;
-          rescaled = true;
-          m = m_new;
         }
         const float2 nm2 = make_float2(kPShift - m, kPShift - m);
-        if constexpr (kFp8PV) {
-          uint32_t pk[16];
-          if (!full) {                               // the ragged last tile: masked keys give 0
+        float2 ac[4];
 #pragma unroll
-            for (int c = 0; c < 64; ++c)
-              if (half * 64 + c >= valid) sv[c] = __float_as_uint(-INFINITY);
-          }
+        for (int i = 0; i < 4; ++i) ac[i] = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+        for (int c = c0; c < c1; ++c) {
+          uint32_t sv[32], pk[16], ov = 0;
+          FK_TMEM_LD32(tS + c * 32, sv);
+          FK_TMEM_WAIT_LD32(sv);
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            const float2 x0 = ffma2(make_float2(__uint_as_float(sv[4 * q]), __uint_as_float(sv[4 * q + 1])),
-                                    sc2, nm2);
-            const float2 x1 = ffma2(make_float2(__uint_as_float(sv[4 * q + 2]), __uint_as_float(sv[4 * q + 3])),
-                                    sc2, nm2);
-            float2 e0, e1;
-            e0.x = fast_exp2(x0.x);
-            e0.y = fast_exp2(x0.y);
-            e1.x = fast_exp2(x1.x);
-            e1.y = fast_exp2(x1.y);
-            acc[(2 * q) & 3] = fadd2(acc[(2 * q) & 3], e0);
-            acc[(2 * q + 1) & 3] = fadd2(acc[(2 * q + 1) & 3], e1);
-            pk[q] = e4m3x2(e0.x, e0.y) | (e4m3x2(e1.x, e1.y) << 16);
-          }
-          FK_TMEM_ST16(tS + half * 16, pk);
-          continue;
+          for (int i = 0; i < 32; ++i)               // the ragged last tile: masked keys give 0
+            if (c * 32 + i >= valid) sv[i] = __float_as_uint(-INFINITY);
+          exp_chunk<kFp8PV>(sv, sc2, nm2, ac, pk, ov);
+          if constexpr (kFp8PV) FK_TMEM_ST8(tS + c * 8, pk);
+          else FK_TMEM_ST16(tS + c * 16, pk);
         }
-        uint32_t pk[32];
-        if (full) {
+        const float2 a4 = fadd2(fadd2(ac[0], ac[1]), fadd2(ac[2], ac[3]));
+        l += a4.x + a4.y;
+        return true;
+      };
+      auto hand_over = [&](uint64_t* b) {            // P in TMEM -> the MMA warp
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b);
+      };
+      if (valid >= kAttnBN && j > 0) {               // uniform over the CTA
+        constexpr int kW = kFp8PV ? 8 : 16;          // P words of 32 columns
+        uint32_t ca[32], cb[32], pk[3 * kW], ov = 0;
+        float2 ah[4];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const float2 x = ffma2(make_float2(__uint_as_float(sv[2 * q]), __uint_as_float(sv[2 * q + 1])),
-                                   sc2, nm2);
-            float2 e;
-            e.x = fast_exp2(x.x);                    // MUFU
-            e.y = fast_exp2(x.y);
-            acc[q & 3] = fadd2(acc[q & 3], e);
-            pk[q] = pack_bf16(e.x, e.y);
+        for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
+        float2 nm2 = make_float2(kPShift - m, kPShift - m);
+        FK_TMEM_LD32(tS, ca);
+        FK_TMEM_WAIT_LD32(ca);
+        FK_TMEM_LD32(tS + 32, cb);
+        exp_chunk<kFp8PV>(ca, sc2, nm2, ah, pk, ov);
+        FK_TMEM_WAIT_LD32(cb);
+        FK_TMEM_LD32(tS + 64, ca);
+        exp_chunk<kFp8PV>(cb, sc2, nm2, ah, pk + kW, ov);
+        FK_TMEM_WAIT_LD32(ca);
+        FK_TMEM_LD32(tS + 96, cb);
+        exp_chunk<kFp8PV>(ca, sc2, nm2, ah, pk + 2 * kW, ov);
+        FK_TMEM_WAIT_LD32(cb);
+        if (!exceeds<kFp8PV>(ah, ov)) {              // warp-uniform
+          if constexpr (kFp8PV) {
+            FK_TMEM_ST16(tS, pk);
+            FK_TMEM_ST8(tS + 16, (pk + 16));
+          } else {
+            FK_TMEM_ST32(tS, pk);
+            FK_TMEM_ST16(tS + 32, (pk + 32));
           }
-        } else {
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const int c = half * 64 + 2 * q;
-            const float x0 = c < valid ? __uint_as_float(sv[2 * q]) : -INFINITY;
-            const float x1 = c + 1 < valid ? __uint_as_float(sv[2 * q + 1]) : -INFINITY;
-            float2 e;
-            e.x = fast_exp2(fmaf(x0, sl2, -m));
-            e.y = fast_exp2(fmaf(x1, sl2, -m));
-            acc[q & 3] = fadd2(acc[q & 3], e);
-            pk[q] = pack_bf16(e.x, e.y);
-          }
+          const float2 a4 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
+          l += a4.x + a4.y;
+        } else if (!general_part(0, 3)) {
+          ok = false;
+          break;
         }
-        FK_TMEM_ST32(tS + half * 32, pk);
+        hand_over(&bar->pa_full[t]);
+        nm2 = make_float2(kPShift - m, kPShift - m);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
+        ov = 0;
+        exp_chunk<kFp8PV>(cb, sc2, nm2, ah, pk, ov);
+        if (!exceeds<kFp8PV>(ah, ov)) {
+          if constexpr (kFp8PV) FK_TMEM_ST8(tS + 24, pk);
+          else FK_TMEM_ST16(tS + 48, pk);
+          const float2 a4 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
+          l += a4.x + a4.y;
+        } else if (!general_part(3, 4)) {
+          ok = false;
+          break;
+        }
+      } else {
+        if (!general_part(0, 3)) { ok = false; break; }
+        hand_over(&bar->pa_full[t]);
+        if (!general_part(3, 4)) { ok = false; break; }
       }
-      const float2 acc01 = fadd2(acc[0], acc[1]), acc23 = fadd2(acc[2], acc[3]);
-      const float2 acc4 = fadd2(acc01, acc23);
-      l += acc4.x + acc4.y;
-      if (rescaled && j > 0) {                       // PV_t(j-1) is complete (see MMA order)
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t o[32];
-          FK_TMEM_LD32(tO + c * 32, o);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha_tile);
-          FK_TMEM_ST32(tO + c * 32, o);
-        }
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar->p_full[t]);
+      hand_over(&bar->p_full[t]);
     }
     // ---------------------------------------------------------------- epilogue
     if (kSplit && ok && warp_wait(&bar->o_done, 0, bar, a.status)) {

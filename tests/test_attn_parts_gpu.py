@@ -1,0 +1,40 @@
+"""Attention: the running maximum raised in either part of a key tile (keys 0-95 and 96-127 are
+handed to the tensor cores separately), in the first, a middle and the ragged last tile."""
+import numpy as np
+import pytest
+
+import workloads as W
+from fkharness import run_snapshot
+
+pytestmark = pytest.mark.gpu
+
+
+def _spiked(w, spikes, seed):
+    """Snapshot inputs whose queries share a direction u, and keys a * u at the given positions of
+    the head's key set [current chunk | sink | anchor]: logits of about 22.6 a (D = 128)."""
+    rng = np.random.default_rng(seed)
+    F, H, D = w.tokens_per_frame, w.n_heads, w.head_dim
+    u = rng.choice([-1.0, 1.0], size=D)
+    K = rng.standard_normal((3 * F, H, D))
+    V = rng.standard_normal((3 * F, H, D))
+    for pos, a in spikes:
+        K[pos] = a * u
+    q = rng.standard_normal((F, H, D)) + 2.0 * u
+    b = W.to_bf16_bits
+    return b(K[F:]), b(V[F:]), b(K[:F]), b(V[:F]), b(q)
+
+
+@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+@pytest.mark.parametrize("tokens", [384, 404, 418])       # last tile full, 60 keys, 102 keys
+def test_maximum_raised_in_either_part(dim, precision, tokens):
+    w = W.TINY_PER_FRAME.with_(name="parts", n_heads=2, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
+                               n_sink_frames=1, n_history_frames=2, n_segments=2, static_heads=(0, 1),
+                               attn_precision=precision)
+    nk = 3 * tokens
+    last = (nk - 1) // 128 * 128
+    # part 2 of the first tile, part 1 and part 2 of middle tiles, both parts of one tile, the
+    # last tile; each above the one before (0.25 is ~8 in log2 units)
+    spikes = [(100, 0.25), (128 + 40, 0.5), (256 + 120, 0.75), (512 + 3, 1.0), (512 + 127, 1.5),
+              (last + 5, 2.0), (nk - 1, 2.5)]
+    for n in range(len(spikes) + 1):           # the maximum stays at each of them once
+        run_snapshot(w, inputs=_spiked(w, spikes[:n], seed=n))
