@@ -89,6 +89,8 @@ struct Layout {
   static constexpr int kOffQ16 = kOffV + 2 * kKV; // FP8: two bf16 query tiles
   static constexpr int kOffBar = kOffQ16 + 2 * kQ16;
   static constexpr int kUsed = kOffBar + 256;
+  // the key splits' merge: R = ceil(256 / splits) rows of O and (m, l) from every split
+  static_assert((2 * kAttnBM + kMaxKvSplits - 1) * (D * 4 + 8) <= kOffBar, "merge space");
   // at least ~116 KB so that one CTA occupies an SM (its 512 TMEM columns are then free)
   static constexpr int kSmem = (kUsed + 1024) > 118 * 1024 ? (kUsed + 1024) : 118 * 1024;
 };
@@ -302,6 +304,24 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// barrier over every thread of the cluster (release / acquire)
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// shared-memory address of CTA `rank` of the cluster, and stores to such an address
+__device__ __forceinline__ uint32_t map_peer(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, uint4 v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" :: "r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+
 // packed fp32 pair arithmetic (sm_100+): two lanes of work per instruction
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   float2 d;
@@ -374,8 +394,8 @@ __device__ __forceinline__ bool exceeds(const float2* ah, uint32_t ov) {
   return __any_sync(0xffffffffu, hs2.x + hs2.y > 256.0f);
 }
 
-// kSplit: a launch with key splits (kv_splits > 1); the unsplit instantiation carries none of
-// the split bookkeeping.  kFp8: Q K^T on E4M3 operands (D = 128).  kFp8PV (with kFp8): P V on
+// kSplit: a launch with key splits (kv_splits > 1): the splits of one pair of query tiles are the
+// CTAs of a cluster, merged at the end through distributed shared memory.  kFp8: Q K^T on E4M3 operands (D = 128).  kFp8PV (with kFp8): P V on
 // E4M3 operands too: V tiles from the E4M3 copy of the V view arena (one 128-byte swizzle atom
 // per key row), P written as e4m3 of 2^6 exp2(s c - m), four keys per TMEM column.
 template <int D, bool kSplit, bool kFp8, bool kFp8PV = false>
@@ -499,6 +519,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       }
     }
     __syncwarp();
+    if constexpr (kSplit) {                        // the merge's two barriers
+      cluster_sync();
+      cluster_sync();
+    }
   } else if (warp == kWarpMma) {
     // ------------------------------------------------------------------ MMA issuer
     // Order per key tile j:  PV0(j), S0(j+1), PV1(j), S1(j+1).  Tensor-core operations of
@@ -581,6 +605,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
     wait_phase(&bar->fin, 0, bar, a.status, false);
     __syncwarp();
+    if constexpr (kSplit) {
+      cluster_sync();
+      cluster_sync();
+    }
   } else {
     // ------------------------------------------------------------------ softmax warpgroups
     const int t = warp >> 2;                        // query tile of this warpgroup
@@ -760,25 +788,70 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       hand_over(&bar->p_full[t]);
     }
     // ---------------------------------------------------------------- epilogue
-    if (kSplit && ok && warp_wait(&bar->o_done, 0, bar, a.status)) {
-      // one key split: unnormalised O and the row's (m, l), merged by merge_kernel
+    if constexpr (kSplit) {
+      // Merge of the key splits through distributed shared memory.  CTA r of the cluster merges
+      // rows [r R, (r + 1) R) of the 256: every thread sends its row of unnormalised O and the row's
+      // (m, l) to the row's owner, whose operand tiles are free once every CTA's MMAs are done
+      // (16-byte chunk c of row i at chunk c ^ (i mod D/4): a warp's rows then hit distinct
+      // banks); the owner forms O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s, M = max_s m_s.
+      const int S = a.kv_splits, R = (2 * kAttnBM + S - 1) / S;
+      const int grow = t * kAttnBM + row, owner = grow / R, lr = grow - owner * R;
+      float2* ml = reinterpret_cast<float2*>(smem + S * R * D * 4);
+      ok = ok && warp_wait(&bar->o_done, 0, bar, a.status);
       tc_fence_after();
-      const int q = q0 + t * kAttnBM + row;
-      const int64_t slot = ((int64_t)split * a.Nq + q) * a.H + head;
-      float* prow = a.part_o + slot * D;
+      cluster_sync();                               // every CTA is done with its operand tiles
+      if (ok) {
+        const uint32_t slot = (uint32_t)(split * R + lr);
+        const uint32_t dst = map_peer(su32(smem) + slot * (D * 4), owner);
 #pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t o[32];
-        FK_TMEM_LD32(tO + c * 32, o);
-        tmem_wait_ld();
-        if (q < a.Nq) {
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t o[32];
+          FK_TMEM_LD32(tO + c * 32, o);
+          FK_TMEM_WAIT_LD32(o);
 #pragma unroll
-          for (int e = 0; e < 32; e += 4)
-            *reinterpret_cast<uint4*>(prow + c * 32 + e) = make_uint4(o[e], o[e + 1], o[e + 2], o[e + 3]);
+          for (int e = 0; e < 8; ++e)
+            st_peer(dst + (uint32_t)(((c * 8 + e) ^ (lr & (D / 4 - 1))) * 16),
+                    make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]));
         }
+        st_peer(map_peer(su32(ml + slot), owner), make_float2(m, l));
       }
-      if (q < a.Nq) a.part_ml[slot] = make_float2(m, l);
-    } else if (!kSplit && ok && warp_wait(&bar->o_done, 0, bar, a.status)) {
+      cluster_sync();                               // every row has arrived
+      // D / 8 lanes per row, eight channels each
+      constexpr int kLanes = D / 8;
+      const int cl = lane % kLanes;
+      const int rows = min(R, 2 * kAttnBM - split * R);
+      for (int r = warp * (32 / kLanes) + lane / kLanes; r < rows; r += 8 * (32 / kLanes)) {
+        const int q = q0 + split * R + r;
+        if (q >= a.Nq) break;
+        float M = -INFINITY;
+        for (int sp = 0; sp < S; ++sp) M = fmaxf(M, ml[sp * R + r].x);
+        float L = 0.0f, acc[8];
+#pragma unroll
+        for (int d = 0; d < 8; ++d) acc[d] = 0.0f;
+        for (int sp = 0; sp < S; ++sp) {
+          const float2 x = ml[sp * R + r];
+          const float w = fast_exp2(x.x - M);
+          const float4* src = reinterpret_cast<const float4*>(smem + (sp * R + r) * (D * 4));
+          const float4 lo = src[(2 * cl) ^ (r & (D / 4 - 1))], hi4 = src[(2 * cl + 1) ^ (r & (D / 4 - 1))];
+          L = fmaf(w, x.y, L);
+          acc[0] = fmaf(w, lo.x, acc[0]);
+          acc[1] = fmaf(w, lo.y, acc[1]);
+          acc[2] = fmaf(w, lo.z, acc[2]);
+          acc[3] = fmaf(w, lo.w, acc[3]);
+          acc[4] = fmaf(w, hi4.x, acc[4]);
+          acc[5] = fmaf(w, hi4.y, acc[5]);
+          acc[6] = fmaf(w, hi4.z, acc[6]);
+          acc[7] = fmaf(w, hi4.w, acc[7]);
+        }
+        const float inv = 1.0f / L;
+        uint4 v;
+        v.x = pack_bf16(acc[0] * inv, acc[1] * inv);
+        v.y = pack_bf16(acc[2] * inv, acc[3] * inv);
+        v.z = pack_bf16(acc[4] * inv, acc[5] * inv);
+        v.w = pack_bf16(acc[6] * inv, acc[7] * inv);
+        *reinterpret_cast<uint4*>(a.O + ((int64_t)q * a.H + head) * D + cl * 8) = v;
+      }
+    } else if (ok && warp_wait(&bar->o_done, 0, bar, a.status)) {
       tc_fence_after();
       const float inv = 1.0f / l;
       const int q = q0 + t * kAttnBM + row;
@@ -1111,47 +1184,6 @@ cudaError_t launch_head_profile(int head_dim, const CUtensorMap& tmQ, const CUte
   return cudaGetLastError();
 }
 
-namespace {
-
-// Merge of the key splits of one query row and head (one warp): with M = max_s m_s (log2
-// domain), O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s, stored as bf16.
-template <int D>
-__global__ void __launch_bounds__(256) merge_kernel(const float* part_o, const float2* part_ml,
-                                                    bf16* O, int Nq, int H, int splits) {
-  constexpr int kPer = D / 32;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= (int64_t)Nq * H) return;
-  float M = -INFINITY;
-  for (int sp = 0; sp < splits; ++sp) M = fmaxf(M, part_ml[sp * (int64_t)Nq * H + w].x);
-  float L = 0.0f, acc[kPer];
-#pragma unroll
-  for (int d = 0; d < kPer; ++d) acc[d] = 0.0f;
-  for (int sp = 0; sp < splits; ++sp) {
-    const int64_t slot = sp * (int64_t)Nq * H + w;
-    const float2 ml = part_ml[slot];
-    const float wgt = fast_exp2(ml.x - M);
-    L = fmaf(wgt, ml.y, L);
-    const float* src = part_o + slot * D + lane * kPer;
-#pragma unroll
-    for (int d = 0; d < kPer; ++d) acc[d] = fmaf(wgt, src[d], acc[d]);
-  }
-  const float inv = 1.0f / L;
-  bf16* dst = O + w * D + lane * kPer;
-#pragma unroll
-  for (int d = 0; d < kPer; d += 2)
-    *reinterpret_cast<uint32_t*>(dst + d) = pack_bf16(acc[d] * inv, acc[d + 1] * inv);
-}
-
-}  // namespace
-
-void launch_merge(int head_dim, const AttnArgs& a, cudaStream_t s) {
-  const int64_t warps = (int64_t)a.Nq * a.H;
-  const unsigned grid = (unsigned)((warps * 32 + 255) / 256);
-  if (head_dim == 128) merge_kernel<128><<<grid, 256, 0, s>>>(a.part_o, a.part_ml, a.O, a.Nq, a.H, a.kv_splits);
-  else merge_kernel<64><<<grid, 256, 0, s>>>(a.part_o, a.part_ml, a.O, a.Nq, a.H, a.kv_splits);
-}
-
 cudaError_t attention_prepare(int head_dim) {
   const auto set = [](const void* fn, int smem) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1170,35 +1202,59 @@ cudaError_t attention_prepare(int head_dim) {
   return set((const void*)attn_kernel<64, true, false>, Layout<64>::kSmem);
 }
 
-void launch_attention(int head_dim, int precision, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                      const CUtensorMap& tmV, const AttnArgs& a, cudaStream_t s) {
-  using Kern = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
-  const bool split = a.kv_splits > 1;
-  Kern kern;
-  int smem;
+namespace {
+using AttnKern = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
+AttnKern attention_kernel(int head_dim, int precision, bool split, int* smem) {
   if (head_dim == 128 && precision == FK_ATTN_FP8) {
-    kern = split ? attn_kernel<128, true, true, true> : attn_kernel<128, false, true, true>;
-    smem = Layout<128, true, true>::kSmem;
-  } else if (head_dim == 128 && precision == FK_ATTN_FP8_QK) {
-    kern = split ? attn_kernel<128, true, true> : attn_kernel<128, false, true>;
-    smem = Layout<128, true>::kSmem;
-  } else if (head_dim == 128) {
-    kern = split ? attn_kernel<128, true, false> : attn_kernel<128, false, false>;
-    smem = Layout<128>::kSmem;
-  } else {
-    kern = split ? attn_kernel<64, true, false> : attn_kernel<64, false, false>;
-    smem = Layout<64>::kSmem;
+    *smem = Layout<128, true, true>::kSmem;
+    return split ? attn_kernel<128, true, true, true> : attn_kernel<128, false, true, true>;
   }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(a.n_qtiles * a.H * a.kv_splits));
-  cfg.blockDim = dim3(kAttnThreads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  if (head_dim == 128 && precision == FK_ATTN_FP8_QK) {
+    *smem = Layout<128, true>::kSmem;
+    return split ? attn_kernel<128, true, true> : attn_kernel<128, false, true>;
+  }
+  if (head_dim == 128) {
+    *smem = Layout<128>::kSmem;
+    return split ? attn_kernel<128, true, false> : attn_kernel<128, false, false>;
+  }
+  *smem = Layout<64>::kSmem;
+  return split ? attn_kernel<64, true, false> : attn_kernel<64, false, false>;
+}
+// launch configuration with programmatic dependent launch and, for key splits, a cluster of them
+void attention_config(int splits, int grid, int smem, cudaStream_t s, cudaLaunchConfig_t* cfg,
+                      cudaLaunchAttribute* attr) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)grid);
+  cfg->blockDim = dim3(kAttnThreads);
+  cfg->dynamicSmemBytes = (size_t)smem;
+  cfg->stream = s;
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)splits;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = splits > 1 ? 2 : 1;
+}
+}  // namespace
+
+cudaError_t attention_clusters(int head_dim, int precision, int splits, int* n) {
+  int smem;
+  const AttnKern kern = attention_kernel(head_dim, precision, true, &smem);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  attention_config(splits, splits, smem, nullptr, &cfg, attr);
+  return cudaOccupancyMaxActiveClusters(n, kern, &cfg);
+}
+
+void launch_attention(int head_dim, int precision, const CUtensorMap& tmQ, const CUtensorMap& tmK,
+                      const CUtensorMap& tmV, const AttnArgs& a, cudaStream_t s) {
+  int smem;
+  const AttnKern kern = attention_kernel(head_dim, precision, a.kv_splits > 1, &smem);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  attention_config(a.kv_splits, a.n_qtiles * a.H * a.kv_splits, smem, s, &cfg, attr);
   cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, a);
 }
 

@@ -14,8 +14,7 @@
 //                frame f lives in slot f (f < S) or S + (f - S) mod cap_nonsink.
 //   scores       fp32 [target][ring_slots][n]; kept lists int32 [target][kmax];
 //                int64 scoring sums (scratch); status word;
-//                host staging (two slots of K, V and Q; O) and the attention key-split
-//                scratch (fp32 partial outputs and row statistics of two splits).
+//                host staging (two slots of K, V and Q; O).
 //   FP8 only     the E4M3 copy of the K view arena ([rows][D] bytes, written by the copy
 //                kernels together with every bf16 view K row) and, when P V also runs on
 //                E4M3 (FK_ATTN_FP8), of the V view arena; the attention kernel quantizes
@@ -99,35 +98,42 @@ bool get_encode() {
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// Key splits of one attention launch.  The CTAs (one per SM) are dispatched longest first;
-// the makespan on n_sms SMs is estimated greedily in units of key tiles (plus a fixed cost
-// per CTA), without and with 2 key splits (plus the merge pass); equal-length heads whose CTAs
-// fill 1.5 waves are where the split pays.
-int choose_kv_splits(int n_sms, int n_qtiles, int CF, int H, int D, const int* n_keys) {
-  const double kOverheadTiles = 3.0, kTileUs = 1.65, kHbmBytesPerUs = 6.0e6;
-  auto makespan = [&](int sp) {
-    std::vector<double> d;
-    for (int hd = 0; hd < H; ++hd) {
-      const int nt = (n_keys[hd] + kAttnBN - 1) / kAttnBN;
-      if (nt < sp) return 1e30;
-      for (int q = 0; q < n_qtiles; ++q)
-        for (int k = 0; k < sp; ++k) d.push_back((double)((k + 1) * nt / sp - k * nt / sp) + kOverheadTiles);
-    }
-    std::sort(d.begin(), d.end(), std::greater<double>());
+// Key splits of one attention launch.  The CTAs (one per SM) are dispatched longest first; the
+// makespan is estimated greedily in units of key tiles for every split count: a cluster of k CTAs
+// takes ceil(tiles / k) tiles and a fixed cost (set-up, first loads, epilogue, and with k > 1 the
+// merge), on the `clusters[k]` clusters that the device holds at once.  Grids that leave SMs idle
+// (few heads or queries) or whose last wave is short are where splits pay.  Measured, k = 1 / best
+// (k chosen): 6 heads, 808 queries, 2828 and 2020 keys 38 / 21 us (5); 4 heads, 2412 queries,
+// 13132 and 4020 keys 135 / 48 us (4); 12 heads, 4680 queries, 15600 keys 328 / 293 us (2), 25480
+// and 7800 keys 286 us (1; 320 us with 2).  The overheads are fitted to such sweeps of k.
+int choose_kv_splits(const int* clusters, int n_qtiles, int H, const int* n_keys) {
+  const double kOverheadTiles = 3.5, kMergeTiles = 2.5;
+  int tiles[kMaxHeads], min_tiles = 1 << 30;
+  for (int hd = 0; hd < H; ++hd) {
+    tiles[hd] = (n_keys[hd] + kAttnBN - 1) / kAttnBN;
+    min_tiles = std::min(min_tiles, tiles[hd]);
+  }
+  std::sort(tiles, tiles + H, std::greater<int>());
+  int best = 1;
+  double best_span = 0.0;
+  for (int k = 1; k <= std::min(kMaxKvSplits, min_tiles); ++k) {
+    if (clusters[k] < 1) continue;
     std::priority_queue<double, std::vector<double>, std::greater<double>> load;
-    for (int i = 0; i < n_sms; ++i) load.push(0.0);
+    for (int i = 0; i < clusters[k]; ++i) load.push(0.0);
     double span = 0.0;
-    for (double x : d) {
-      const double t = load.top() + x;
-      load.pop();
-      load.push(t);
-      span = std::max(span, t);
+    for (int hd = 0; hd < H; ++hd)
+      for (int q = 0; q < n_qtiles; ++q) {
+        const double t = load.top() + (tiles[hd] + k - 1) / k + kOverheadTiles + (k > 1 ? kMergeTiles : 0.0);
+        load.pop();
+        load.push(t);
+        span = std::max(span, t);
+      }
+    if (k == 1 || span < 0.97 * best_span) {
+      best = k;
+      best_span = span;
     }
-    return span;
-  };
-  const double merge_tiles =
-      ((double)kMaxKvSplits * CF * H * D * 4 + (double)CF * H * D * 2) / kHbmBytesPerUs / kTileUs;
-  return makespan(2) + merge_tiles < 0.95 * makespan(1) ? 2 : 1;
+  }
+  return best;
 }
 
 }  // namespace
@@ -170,10 +176,8 @@ struct fk_handle {
   int64_t stage_frames = 0;        // frames one K/V staging buffer holds
   cudaStream_t copy_stream = nullptr;
   bool host_overlap = false;
-  // attention key splits: scratch for split outputs, SM count, last decision per layer
-  float* part_o = nullptr;
-  float2* part_ml = nullptr;
-  int n_sms = 0;
+  // attention key splits: clusters resident at once per split count, last decision per layer
+  int attn_clusters[kMaxKvSplits + 1] = {};
   std::vector<std::vector<int>> split_keys;   // [L]: key counts the cached decision was made for
   std::vector<int> split_choice;              // [L]
   ScoreItem* d_score_items = nullptr;
@@ -849,16 +853,15 @@ fk_status fk_create(const fk_config* cfg, fk_handle** out) {
       return fail(FK_ERR_CUDA);
     }
   }
-  if ((st = dev_alloc(h, (size_t)kMaxKvSplits * h->CF * h->H * h->D * sizeof(float), &p)) != FK_OK)
-    return fail(st);
-  h->part_o = static_cast<float*>(p);
-  if ((st = dev_alloc(h, (size_t)kMaxKvSplits * h->CF * h->H * sizeof(float2), &p)) != FK_OK)
-    return fail(st);
-  h->part_ml = static_cast<float2*>(p);
-  if (cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->dev) != cudaSuccess) {
+  if (cudaDeviceGetAttribute(&h->attn_clusters[1], cudaDevAttrMultiProcessorCount, h->dev) != cudaSuccess) {
     cudaGetLastError();
     return fail(FK_ERR_CUDA);
   }
+  for (int k = 2; k <= kMaxKvSplits; ++k)
+    if (attention_clusters(h->D, h->precision, k, &h->attn_clusters[k]) != cudaSuccess) {
+      cudaGetLastError();
+      h->attn_clusters[k] = 0;
+    }
   h->split_keys.assign(h->L, {});
   h->split_choice.assign(h->L, 1);
   h->stage_frames = h->C;
@@ -1208,12 +1211,10 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
   for (int i = 0; i < h->H; ++i) a.head_of[i] = order[i];
   std::vector<int> keys(a.n_keys, a.n_keys + h->H);
   if (keys != h->split_keys[layer]) {
-    h->split_choice[layer] = choose_kv_splits(h->n_sms, a.n_qtiles, h->CF, h->H, h->D, a.n_keys);
+    h->split_choice[layer] = choose_kv_splits(h->attn_clusters, a.n_qtiles, h->H, a.n_keys);
     h->split_keys[layer] = keys;
   }
   a.kv_splits = h->split_choice[layer];
-  a.part_o = h->part_o;
-  a.part_ml = h->part_ml;
   const int D = h->D;
   // FP8: the E4M3 keys (and, for P V, values) come from the view arenas' E4M3 copies; the kernel
   // quantizes Q
@@ -1221,10 +1222,8 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
   const CUtensorMap& tv = h->fp8pv ? h->tmV8 : h->tmV;
   if ((st = launch(h, s, FK_KERNEL_ATTEND, [&] {
          launch_attention(D, h->precision, h->tmQ[qm], tk, tv, a, s);
-         if (a.kv_splits > 1) launch_merge(D, a, s);
        })) != FK_OK)
     return st;
-  if (a.kv_splits > 1) h->launches++;   // the merge pass
   if (slot >= 0) FK_CUDA(cudaEventRecord(h->st_q.freed[slot], s));
   if (copy_back) {
     if (h->host_overlap) {   // copy back off the caller's stream; fk_wait_outputs joins it

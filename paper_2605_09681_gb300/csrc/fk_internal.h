@@ -19,6 +19,7 @@ constexpr int kMaxHeads = 128;
 constexpr int kMaxLayers = 256;
 constexpr int kAttnBM = 128;          // query rows per attention CTA
 constexpr int kAttnBN = 128;          // keys per attention tile
+constexpr int kMaxKvSplits = 8;       // key splits of one attention CTA (the portable cluster size)
 constexpr int kViewAlignRows = 128;   // packed views are padded to whole key tiles
 // scoring CTA: 4 warps; a token is owned by 4 lanes, so a CTA covers 32 tokens of a segment
 // (one frame-chunk)
@@ -248,9 +249,8 @@ struct AttnArgs {
   int n_qtiles;
   float scale_log2;             // log2(e) / sqrt(D)
   int* status;
-  int kv_splits;                // key splits per (head, query-tile pair): 1, or 2 with a merge
-  float* part_o;                // [kv_splits][Nq][H][D] unnormalised split outputs (kv_splits > 1)
-  float2* part_ml;              // [kv_splits][Nq][H] {running max (log2 domain), row sum}
+  int kv_splits;                // key splits per (head, query-tile pair), 1..kMaxKvSplits and at most
+                                // the key tiles of every head: the CTAs of one cluster
   int head_of[kMaxHeads];       // CTA order: head index of the i-th (longest-first) head
   int row_base[kMaxHeads];      // first row of the head's packed view in the view arena
   int n_keys[kMaxHeads];        // keys the head attends to
@@ -263,9 +263,8 @@ struct AttnArgs {
 void launch_attention(int head_dim, int precision, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                       const CUtensorMap& tmV, const AttnArgs& a, cudaStream_t s);
 cudaError_t attention_prepare(int head_dim);   // sets the dynamic shared-memory limits
-// combine the key splits of every (row, head) into O (bf16)
-void launch_merge(int head_dim, const AttnArgs& a, cudaStream_t s);
-constexpr int kMaxKvSplits = 2;
+// clusters of `splits` attention CTAs that the device holds at once
+cudaError_t attention_clusters(int head_dim, int precision, int splits, int* n);
 
 // ------------------------------------------------------------------ FP8 (E4M3) quantization
 // One launch: the query rows (part 0, row-scaled) and key row ranges of a [rows][k_dim] bf16

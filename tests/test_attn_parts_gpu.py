@@ -38,3 +38,15 @@ def test_maximum_raised_in_either_part(dim, precision, tokens):
               (last + 5, 2.0), (nk - 1, 2.5)]
     for n in range(len(spikes) + 1):           # the maximum stays at each of them once
         run_snapshot(w, inputs=_spiked(w, spikes[:n], seed=n))
+
+
+@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+@pytest.mark.parametrize("heads,tokens,sinks", [(1, 171, 1), (1, 256, 1), (1, 277, 1), (1, 341, 1), (2, 170, 1),
+                                                (40, 225, 3), (70, 225, 3), (1, 1040, 1)])
+def test_key_splits(dim, precision, heads, tokens, sinks):
+    """Grids whose heads have 4 to 9 (and 25) key tiles, the last one of 1 to 128 keys: 2 to 8 key
+    splits with uneven ranges, query tiles of 1 to 256 rows."""
+    w = W.TINY_PER_FRAME.with_(name="splits", n_heads=heads, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
+                               n_sink_frames=sinks, n_history_frames=sinks + 1, n_segments=1,
+                               static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
+    run_snapshot(w)
