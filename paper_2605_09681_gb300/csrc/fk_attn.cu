@@ -89,8 +89,7 @@ struct Layout {
   static constexpr int kOffQ16 = kOffV + 2 * kKV; // FP8: two bf16 query tiles
   static constexpr int kOffBar = kOffQ16 + 2 * kQ16;
   static constexpr int kUsed = kOffBar + 256;
-  // the key splits' merge: R = ceil(256 / splits) rows of O and (m, l) from every split
-  static_assert((2 * kAttnBM + kMaxKvSplits - 1) * (D * 4 + 8) <= kOffBar, "merge space");
+  static_assert(2 * kAttnBM * (D * 4 + 8) <= kOffBar, "the key splits' rows of O and their (m, l)");
   // at least ~116 KB so that one CTA occupies an SM (its 512 TMEM columns are then free)
   static constexpr int kSmem = (kUsed + 1024) > 118 * 1024 ? (kUsed + 1024) : 118 * 1024;
 };
@@ -308,18 +307,22 @@ __device__ __forceinline__ float fast_exp2(float x) {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// shared-memory address of CTA `rank` of the cluster, and stores to such an address
+// shared-memory address of CTA `rank` of the cluster, and loads from such an address
 __device__ __forceinline__ uint32_t map_peer(uint32_t addr, int rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_peer(uint32_t addr, uint4 v) {
-  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "r"(v.x), "r"(v.y),
-               "r"(v.z), "r"(v.w) : "memory");
+__device__ __forceinline__ float4 ld_peer4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
 }
-__device__ __forceinline__ void st_peer(uint32_t addr, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" :: "r"(addr), "f"(v.x), "f"(v.y) : "memory");
+__device__ __forceinline__ float2 ld_peer2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
 }
 
 // packed fp32 pair arithmetic (sm_100+): two lanes of work per instruction
@@ -354,6 +357,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
                  "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]),           \
                  "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])            \
                :: "memory")
+
+// 32-column chunks `first` .. `first` + `count` - 1 of a key tile
+template <int kFirst, int kCount>
+struct Chunks {
+  static constexpr int first = kFirst, count = kCount;
+};
 
 // 32 logits -> numerators exp2(s * sc + nm): their sums in four chains, and P words (bf16 pairs, or
 // four E4M3 codes; `ov` then collects the bits of the overflow test).  The sums and roundings of a
@@ -392,6 +401,68 @@ __device__ __forceinline__ bool exceeds(const float2* ah, uint32_t ov) {
   if constexpr (kE4m3) return __any_sync(0xffffffffu, (ov & 0x80808080u) != 0);
   const float2 hs2 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
   return __any_sync(0xffffffffu, hs2.x + hs2.y > 256.0f);
+}
+
+// Rows [g0, g0 + rows) of the key splits' merge by one of 8 warps: with M = max_s m_s (log2 domain),
+// O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s as bf16, `stride` elements from row to row.  D / 4
+// lanes read a row, 16 bytes each; lane k first forms the S <= kS weights of the warp's k-th row.  A
+// load from a peer takes 600-900 cycles, so kRows row groups of every split are in flight.
+template <int D, int kS, int kRows>
+__device__ __forceinline__ void merge_rows(uint32_t part, uint32_t ml, int S, int g0, int rows, bf16* O, int stride,
+                                           int warp, int lane) {
+  constexpr int kLanes = D / 4, kSub = 32 / kLanes;
+  const int sub = lane / kLanes, li = lane % kLanes;
+  float4 x[kRows][kS];
+  auto load = [&](int i0) {
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int r = ((i0 + i) * 8 + warp) * kSub + sub;
+      const uint32_t addr = part + (uint32_t)((g0 + r) * (D * 4) + li * 16);
+#pragma unroll
+      for (int sp = 0; sp < kS; ++sp)
+        x[i][sp] = r < rows && sp < S ? ld_peer4(map_peer(addr, sp)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+  };
+  load(0);
+  float w[kS];
+  {
+    const int r = ((lane / kSub) * 8 + warp) * kSub + lane % kSub;
+    float2 e[kS];
+    float M = -INFINITY, L = 0.0f;
+#pragma unroll
+    for (int sp = 0; sp < kS; ++sp)
+      e[sp] = r < rows && sp < S ? ld_peer2(map_peer(ml + (uint32_t)((g0 + r) * 8), sp)) : make_float2(-INFINITY, 0.0f);
+#pragma unroll
+    for (int sp = 0; sp < kS; ++sp) M = fmaxf(M, e[sp].x);
+#pragma unroll
+    for (int sp = 0; sp < kS; ++sp) {
+      w[sp] = sp < S ? fast_exp2(e[sp].x - M) : 0.0f;
+      L = fmaf(w[sp], e[sp].y, L);
+    }
+    const float inv = 1.0f / L;
+#pragma unroll
+    for (int sp = 0; sp < kS; ++sp) w[sp] *= inv;
+  }
+#pragma unroll 1
+  for (int i0 = 0; (i0 * 8 + warp) * kSub < rows; i0 += kRows) {
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int r = ((i0 + i) * 8 + warp) * kSub + sub;
+      float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int sp = 0; sp < kS; ++sp) {
+        const float ws = __shfl_sync(0xffffffffu, w[sp], ((i0 + i) * kSub + sub) & 31);
+        acc.x = fmaf(ws, x[i][sp].x, acc.x);
+        acc.y = fmaf(ws, x[i][sp].y, acc.y);
+        acc.z = fmaf(ws, x[i][sp].z, acc.z);
+        acc.w = fmaf(ws, x[i][sp].w, acc.w);
+      }
+      if (r < rows)
+        *reinterpret_cast<uint2*>(O + (int64_t)r * stride + (li ^ ((g0 + r) & (D / 4 - 1))) * 4) =
+            make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+    }
+    load(i0 + kRows);
+  }
 }
 
 // kSplit: a launch with key splits (kv_splits > 1): the splits of one pair of query tiles are the
@@ -437,7 +508,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   }
   const int nt = (nk + kAttnBN - 1) / kAttnBN;
 
-  if (threadIdx.x == 0) {
+  // The TMA warp makes the barriers and starts Q and K tile 0 before the CTA meets (the tensor
+  // memory allocation takes ~1000 cycles).
+  constexpr int kQBytes = kAttnBM * D * 2;
+  auto load_k = [&](int j, uint64_t* b) {             // key tile j into K stage j mod 2
+    const int st = j & 1;
+    if constexpr (kFp8) {
+      tma_load_2d(sK + st * Lay::kK, &tmK, b, 0, row0 + j * kAttnBN);
+    } else {
+      for (int h = 0; h < kHalves; ++h)
+        tma_load_2d(sK + st * Lay::kK + h * 16384, &tmK, b, h * 64, row0 + j * kAttnBN);
+    }
+  };
+  if (warp == kWarpTma && lane == 0) {
     mbar_init(&bar->q_full, 1);
     mbar_init(&bar->k0_full, 1);
     mbar_init(&bar->k0_empty, 1);
@@ -454,7 +537,18 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (kFp8) mbar_init(&bar->q8_ready, 2 * kAttnBM);
     bar->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // Q, K and V may have been written by the previous kernel of the stream
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // bf16 query tiles: the MMA operand, or (FP8) the softmax threads' quantization input
+    uint8_t* q_dst = kFp8 ? sQ16 : sQ;
+    mbar_expect_tx(&bar->q_full, 2 * kQBytes);
+    for (int t = 0; t < 2; ++t)
+      for (int h = 0; h < kHalves; ++h)
+        tma_load_3d(q_dst + t * kQBytes + h * 16384, &tmQ, &bar->q_full, h * 64, head, q0 + t * kAttnBM);
+    mbar_expect_tx(&bar->k0_full, Lay::kK);
+    load_k(0, &bar->k0_full);
   }
+  __syncwarp();
   if (warp == kWarpMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(su32(&bar->tmem_base)), "r"(kTmemCols) : "memory");
@@ -469,30 +563,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int lastVK[2] = {-1, -1};
-      bool ok = true, k0 = false;
-      // Q, K and V may have been written by the previous kernel of the stream
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      // bf16 query tiles: the MMA operand, or (FP8) the softmax threads' quantization input
-      uint8_t* q_dst = kFp8 ? sQ16 : sQ;
-      constexpr int kQBytes = kAttnBM * D * 2;
-      mbar_expect_tx(&bar->q_full, 2 * kQBytes);
-      for (int t = 0; t < 2; ++t)
-        for (int h = 0; h < kHalves; ++h)
-          tma_load_3d(q_dst + t * kQBytes + h * 16384, &tmQ, &bar->q_full, h * 64, head,
-                      q0 + t * kAttnBM);
-      auto load_k = [&](int j, uint64_t* b) {         // key tile j into K stage j mod 2
-        const int st = j & 1;
-        if constexpr (kFp8) {
-          tma_load_2d(sK + st * Lay::kK, &tmK, b, 0, row0 + j * kAttnBN);
-        } else {
-          for (int h = 0; h < kHalves; ++h)
-            tma_load_2d(sK + st * Lay::kK + h * 16384, &tmK, b, h * 64, row0 + j * kAttnBN);
-        }
-      };
-      mbar_expect_tx(&bar->k0_full, Lay::kK);
-      load_k(0, &bar->k0_full);
-      k0 = true;
-      // then per key tile j: V_j together with K_{j+1} on one barrier (b = j mod 2).  Their
+      bool ok = true;
+      // per key tile j: V_j together with K_{j+1} on one barrier (b = j mod 2).  Their
       // stages were last used by V_{j-2} and K_{j-1}, released together by vk_empty[b] after
       // iteration j-2's MMAs (K_2 reuses K_0's stage: k0_empty)
       for (int j = 0; j < nt && ok; ++j) {
@@ -513,7 +585,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       }
       if (!ok) {   // drain every load this thread issued before the CTA exits
         wait_phase(&bar->q_full, 0, bar, a.status, false);
-        if (k0) wait_phase(&bar->k0_full, 0, bar, a.status, false);
+        wait_phase(&bar->k0_full, 0, bar, a.status, false);
         for (int bb = 0; bb < 2; ++bb)
           if (lastVK[bb] >= 0) wait_phase(&bar->vk_full[bb], lastVK[bb] & 1, bar, a.status, false);
       }
@@ -663,26 +735,34 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // tiles after the first, P is computed with the running max m straight away, the next
       // 32 columns' load in flight; a part whose numerators all stay within 2^8 is stored, else it
       // is done again by general_part.
-      // general_part: chunks [c0, c1) with a max pass, and m raised when it grows by more than kThr
-      // (FP8 P V: m is the running max rounded up to an integer).  O_t holds PV of every key before
-      // part c0: with part 0 PV_t(j-1) is complete (see MMA order), with part 1 the keys of part 0
-      // once pva_done says so.
-      auto general_part = [&](int c0, int c1) -> bool {
-        float mx = -INFINITY;
-#pragma unroll 1
-        for (int c = c0; c < c1; ++c) {
-          uint32_t sv[32];
-          FK_TMEM_LD32(tS + c * 32, sv);
-          FK_TMEM_WAIT_LD32(sv);
-          float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      // general_part(Chunks<c0, kN>): chunks c0 .. c0 + kN - 1 with a max pass, and m raised when it grows by
+      // more than kThr (FP8 P V: m is the running max rounded up to an integer).  O_t holds PV of
+      // every key before part c0: with part 0 PV_t(j-1) is complete (see MMA order), with part 1 the
+      // keys of part 0 once pva_done says so.
+      auto general_part = [&](auto chunks) -> bool {
+        constexpr int c0 = decltype(chunks)::first, kN = decltype(chunks)::count;
+        uint32_t sv[kN][32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (c * 32 + i < valid) mxa[i & 3] = fmaxf(mxa[i & 3], __uint_as_float(sv[i]));
-          mx = fmaxf(mx, fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])));
+        for (int c = 0; c < kN; ++c) FK_TMEM_LD32(tS + (c0 + c) * 32, sv[c]);
+#pragma unroll
+        for (int c = 0; c < kN; ++c) FK_TMEM_WAIT_LD32(sv[c]);
+        if (valid < (c0 + kN) * 32) {                // the ragged last tile: masked keys give 0
+#pragma unroll
+          for (int c = 0; c < kN; ++c)
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if ((c0 + c) * 32 + i >= valid) sv[c][i] = __float_as_uint(-INFINITY);
         }
+        float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < kN; ++c)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) mxa[i & 3] = fmaxf(mxa[i & 3], __uint_as_float(sv[c][i]));
+        const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
         const float m_new = fmaxf(m, kFp8PV ? ceilf(mx * sl2) : mx * sl2);
-        if (__any_sync(0xffffffffu, m_new > m + kThr)) {               // warp-uniform
-          float alpha;                               // 0 when m = -inf
+        const bool raise = __any_sync(0xffffffffu, m_new > m + kThr);  // warp-uniform
+        float alpha = 1.0f;                          // 0 when m = -inf
+        if (raise) {
           if constexpr (kFp8PV) {                    // integer references: an exact power of two
             const float dm = m - m_new;
             alpha = (m == -INFINITY || dm < -126.0f) ? 0.0f : pow2f((int)dm);
@@ -691,40 +771,35 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           }
           l *= alpha;
           m = m_new;
-          if (c0 > 0) {
-            if (!warp_wait(&bar->pva_done[t], j & 1, bar, a.status)) return false;
-            tc_fence_after();
-          }
-          if (j > 0 || c0 > 0) {
-#pragma unroll 1
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              FK_TMEM_LD32(tO + c * 32, o);
-              FK_TMEM_WAIT_LD32(o);
-#pragma unroll
-              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              FK_TMEM_ST32(tO + c * 32, o);
-            }
-          }
         }
         const float2 nm2 = make_float2(kPShift - m, kPShift - m);
         float2 ac[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) ac[i] = make_float2(0.0f, 0.0f);
-#pragma unroll 1
-        for (int c = c0; c < c1; ++c) {
-          uint32_t sv[32], pk[16], ov = 0;
-          FK_TMEM_LD32(tS + c * 32, sv);
-          FK_TMEM_WAIT_LD32(sv);
 #pragma unroll
-          for (int i = 0; i < 32; ++i)               // the ragged last tile: masked keys give 0
-            if (c * 32 + i >= valid) sv[i] = __float_as_uint(-INFINITY);
-          exp_chunk<kFp8PV>(sv, sc2, nm2, ac, pk, ov);
-          if constexpr (kFp8PV) FK_TMEM_ST8(tS + c * 8, pk);
-          else FK_TMEM_ST16(tS + c * 16, pk);
+        for (int c = 0; c < kN; ++c) {
+          uint32_t pk[16], ov = 0;
+          exp_chunk<kFp8PV>(sv[c], sc2, nm2, ac, pk, ov);
+          if constexpr (kFp8PV) FK_TMEM_ST8(tS + (c0 + c) * 8, pk);
+          else FK_TMEM_ST16(tS + (c0 + c) * 16, pk);
         }
         const float2 a4 = fadd2(fadd2(ac[0], ac[1]), fadd2(ac[2], ac[3]));
         l += a4.x + a4.y;
+        if (raise && (j > 0 || c0 > 0)) {
+          if (c0 > 0) {
+            if (!warp_wait(&bar->pva_done[t], j & 1, bar, a.status)) return false;
+            tc_fence_after();
+          }
+#pragma unroll 1
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t o[32];
+            FK_TMEM_LD32(tO + c * 32, o);
+            FK_TMEM_WAIT_LD32(o);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+            FK_TMEM_ST32(tO + c * 32, o);
+          }
+        }
         return true;
       };
       auto hand_over = [&](uint64_t* b) {            // P in TMEM -> the MMA warp
@@ -733,13 +808,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         __syncwarp();
         if (lane == 0) mbar_arrive(b);
       };
-      if (valid >= kAttnBN && j > 0) {               // uniform over the CTA
-        constexpr int kW = kFp8PV ? 8 : 16;          // P words of 32 columns
-        uint32_t ca[32], cb[32], pk[3 * kW], ov = 0;
-        float2 ah[4];
+      const bool direct = valid >= kAttnBN && j > 0; // uniform over the CTA
+      constexpr int kW = kFp8PV ? 8 : 16;            // P words of 32 columns
+      uint32_t cb[32], ov = 0;
+      float2 ah[4];
+      bool general = true;
+      if (direct) {
+        uint32_t ca[32], pk[3 * kW];
 #pragma unroll
         for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
-        float2 nm2 = make_float2(kPShift - m, kPShift - m);
+        const float2 nm2 = make_float2(kPShift - m, kPShift - m);
         FK_TMEM_LD32(tS, ca);
         FK_TMEM_WAIT_LD32(ca);
         FK_TMEM_LD32(tS + 32, cb);
@@ -751,7 +829,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         FK_TMEM_LD32(tS + 96, cb);
         exp_chunk<kFp8PV>(ca, sc2, nm2, ah, pk + 2 * kW, ov);
         FK_TMEM_WAIT_LD32(cb);
-        if (!exceeds<kFp8PV>(ah, ov)) {              // warp-uniform
+        general = exceeds<kFp8PV>(ah, ov);           // warp-uniform
+        if (!general) {
           if constexpr (kFp8PV) {
             FK_TMEM_ST16(tS, pk);
             FK_TMEM_ST8(tS + 16, (pk + 16));
@@ -761,117 +840,97 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           }
           const float2 a4 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
           l += a4.x + a4.y;
-        } else if (!general_part(0, 3)) {
-          ok = false;
-          break;
         }
-        hand_over(&bar->pa_full[t]);
-        nm2 = make_float2(kPShift - m, kPShift - m);
+      }
+      if (general) {
+        if (!general_part(Chunks<0, 3>{})) { ok = false; break; }
+        if (direct) {                                // (not kept across the general path)
+          FK_TMEM_LD32(tS + 96, cb);
+          FK_TMEM_WAIT_LD32(cb);
+        }
+      }
+      hand_over(&bar->pa_full[t]);
+      general = true;
+      if (direct) {
+        uint32_t pk[kW];
+        const float2 nm2 = make_float2(kPShift - m, kPShift - m);
 #pragma unroll
         for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
         ov = 0;
         exp_chunk<kFp8PV>(cb, sc2, nm2, ah, pk, ov);
-        if (!exceeds<kFp8PV>(ah, ov)) {
+        general = exceeds<kFp8PV>(ah, ov);
+        if (!general) {
           if constexpr (kFp8PV) FK_TMEM_ST8(tS + 24, pk);
           else FK_TMEM_ST16(tS + 48, pk);
           const float2 a4 = fadd2(fadd2(ah[0], ah[1]), fadd2(ah[2], ah[3]));
           l += a4.x + a4.y;
-        } else if (!general_part(3, 4)) {
-          ok = false;
-          break;
         }
-      } else {
-        if (!general_part(0, 3)) { ok = false; break; }
-        hand_over(&bar->pa_full[t]);
-        if (!general_part(3, 4)) { ok = false; break; }
       }
+      if (general && !general_part(Chunks<3, 1>{})) { ok = false; break; }
       hand_over(&bar->p_full[t]);
     }
     // ---------------------------------------------------------------- epilogue
+    // every MMA is done, so the operand tiles' shared memory is free
+    ok = ok && warp_wait(&bar->o_done, 0, bar, a.status);
+    tc_fence_after();
     if constexpr (kSplit) {
-      // Merge of the key splits through distributed shared memory.  CTA r of the cluster merges
-      // rows [r R, (r + 1) R) of the 256: every thread sends its row of unnormalised O and the row's
-      // (m, l) to the row's owner, whose operand tiles are free once every CTA's MMAs are done
-      // (16-byte chunk c of row i at chunk c ^ (i mod D/4): a warp's rows then hit distinct
-      // banks); the owner forms O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s, M = max_s m_s.
-      const int S = a.kv_splits, R = (2 * kAttnBM + S - 1) / S;
-      const int grow = t * kAttnBM + row, owner = grow / R, lr = grow - owner * R;
-      float2* ml = reinterpret_cast<float2*>(smem + S * R * D * 4);
-      ok = ok && warp_wait(&bar->o_done, 0, bar, a.status);
-      tc_fence_after();
-      cluster_sync();                               // every CTA is done with its operand tiles
+      // Merge of the key splits: every CTA of the cluster leaves its 256 rows of unnormalised O (16-
+      // byte chunk c of row g at chunk c ^ (g mod D/4): conflict-free) and their (m, l) in its shared
+      // memory, and CTA r forms rows [r R, (r + 1) R) from all of them, reading whole rows of its
+      // peers.  Bound by the SM-to-SM network, ~13 B per cycle and SM: 128 KB take ~11000 cycles with
+      // 3 splits, as 16-byte stores to the owner took 17500.
+      const int S = a.kv_splits, valid_rows = min(2 * kAttnBM, a.Nq - q0), R = (valid_rows + S - 1) / S;
+      float2* ml = reinterpret_cast<float2*>(smem + 2 * kAttnBM * D * 4);
       if (ok) {
-        const uint32_t slot = (uint32_t)(split * R + lr);
-        const uint32_t dst = map_peer(su32(smem) + slot * (D * 4), owner);
-#pragma unroll
+        const int g = t * kAttnBM + row;
+        uint8_t* dst = smem + g * (D * 4);
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
           FK_TMEM_LD32(tO + c * 32, o);
           FK_TMEM_WAIT_LD32(o);
 #pragma unroll
           for (int e = 0; e < 8; ++e)
-            st_peer(dst + (uint32_t)(((c * 8 + e) ^ (lr & (D / 4 - 1))) * 16),
-                    make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]));
+            *reinterpret_cast<uint4*>(dst + (((c * 8 + e) ^ (g & (D / 4 - 1))) << 4)) =
+                make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
         }
-        st_peer(map_peer(su32(ml + slot), owner), make_float2(m, l));
+        ml[g] = make_float2(m, l);
       }
-      cluster_sync();                               // every row has arrived
-      // D / 8 lanes per row, eight channels each
-      constexpr int kLanes = D / 8;
-      const int cl = lane % kLanes;
-      const int rows = min(R, 2 * kAttnBM - split * R);
-      for (int r = warp * (32 / kLanes) + lane / kLanes; r < rows; r += 8 * (32 / kLanes)) {
-        const int q = q0 + split * R + r;
-        if (q >= a.Nq) break;
-        float M = -INFINITY;
-        for (int sp = 0; sp < S; ++sp) M = fmaxf(M, ml[sp * R + r].x);
-        float L = 0.0f, acc[8];
-#pragma unroll
-        for (int d = 0; d < 8; ++d) acc[d] = 0.0f;
-        for (int sp = 0; sp < S; ++sp) {
-          const float2 x = ml[sp * R + r];
-          const float w = fast_exp2(x.x - M);
-          const float4* src = reinterpret_cast<const float4*>(smem + (sp * R + r) * (D * 4));
-          const float4 lo = src[(2 * cl) ^ (r & (D / 4 - 1))], hi4 = src[(2 * cl + 1) ^ (r & (D / 4 - 1))];
-          L = fmaf(w, x.y, L);
-          acc[0] = fmaf(w, lo.x, acc[0]);
-          acc[1] = fmaf(w, lo.y, acc[1]);
-          acc[2] = fmaf(w, lo.z, acc[2]);
-          acc[3] = fmaf(w, lo.w, acc[3]);
-          acc[4] = fmaf(w, hi4.x, acc[4]);
-          acc[5] = fmaf(w, hi4.y, acc[5]);
-          acc[6] = fmaf(w, hi4.z, acc[6]);
-          acc[7] = fmaf(w, hi4.w, acc[7]);
-        }
-        const float inv = 1.0f / L;
-        uint4 v;
-        v.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-        v.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-        v.z = pack_bf16(acc[4] * inv, acc[5] * inv);
-        v.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-        *reinterpret_cast<uint4*>(a.O + ((int64_t)q * a.H + head) * D + cl * 8) = v;
-      }
-    } else if (ok && warp_wait(&bar->o_done, 0, bar, a.status)) {
-      tc_fence_after();
+      cluster_sync();                               // every CTA's rows are in place
+      const int rows = min(R, valid_rows - split * R);
+      bf16* orow = a.O + ((int64_t)(q0 + split * R) * a.H + head) * D;
+      if (S <= 2) merge_rows<D, 2, 8>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      else if (S <= 4) merge_rows<D, 4, 4>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      else merge_rows<D, 8, 2>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      cluster_sync();                               // every peer has read this CTA's rows
+    } else if (ok) {
+      // normalise, and through the warp's own 32 rows of shared memory (16-byte chunk c of row r at
+      // chunk c ^ (r mod D/8)) to whole rows of O: a thread storing its own row took ~3 us per CTA
       const float inv = 1.0f / l;
-      const int q = q0 + t * kAttnBM + row;
-      bf16* orow = a.O + ((int64_t)q * a.H + head) * D;
-#pragma unroll
+      uint8_t* stage = smem + warp * (32 * D * 2);
+#pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t o[32];
         FK_TMEM_LD32(tO + c * 32, o);
-        tmem_wait_ld();
-        if (q < a.Nq) {
+        FK_TMEM_WAIT_LD32(o);
 #pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            uint4 v;
-            v.x = pack_bf16(__uint_as_float(o[e + 0]) * inv, __uint_as_float(o[e + 1]) * inv);
-            v.y = pack_bf16(__uint_as_float(o[e + 2]) * inv, __uint_as_float(o[e + 3]) * inv);
-            v.z = pack_bf16(__uint_as_float(o[e + 4]) * inv, __uint_as_float(o[e + 5]) * inv);
-            v.w = pack_bf16(__uint_as_float(o[e + 6]) * inv, __uint_as_float(o[e + 7]) * inv);
-            *reinterpret_cast<uint4*>(orow + c * 32 + e) = v;
-          }
+        for (int e = 0; e < 32; e += 8) {
+          uint4 v;
+          v.x = pack_bf16(__uint_as_float(o[e + 0]) * inv, __uint_as_float(o[e + 1]) * inv);
+          v.y = pack_bf16(__uint_as_float(o[e + 2]) * inv, __uint_as_float(o[e + 3]) * inv);
+          v.z = pack_bf16(__uint_as_float(o[e + 4]) * inv, __uint_as_float(o[e + 5]) * inv);
+          v.w = pack_bf16(__uint_as_float(o[e + 6]) * inv, __uint_as_float(o[e + 7]) * inv);
+          *reinterpret_cast<uint4*>(stage + lane * (D * 2) + (((c * 4 + e / 8) ^ (lane & (D / 8 - 1))) << 4)) = v;
         }
+      }
+      __syncwarp();
+      constexpr int kLanes = D / 8;                 // lanes of one row
+      const int cl = lane % kLanes;
+#pragma unroll
+      for (int r0 = 0; r0 < 32; r0 += 32 / kLanes) {
+        const int r = r0 + lane / kLanes, q = q0 + t * kAttnBM + wq * 32 + r;
+        const uint4 v = *reinterpret_cast<const uint4*>(stage + r * (D * 2) + ((cl ^ (r & (D / 8 - 1))) << 4));
+        if (q < a.Nq) *reinterpret_cast<uint4*>(a.O + ((int64_t)q * a.H + head) * D + cl * 8) = v;
       }
     }
   }

@@ -50,3 +50,35 @@ def test_key_splits(dim, precision, heads, tokens, sinks):
                                n_sink_frames=sinks, n_history_frames=sinks + 1, n_segments=1,
                                static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
     run_snapshot(w)
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+def test_key_splits_on_two_streams(dim):
+    """Layers attended on two streams at once (split launches share the handle's exchange slots)
+    give what one stream gives, over many rounds."""
+    import torch
+
+    from paper_2605_09681_gb300 import ForcingKVCache
+    g = torch.Generator(device="cuda").manual_seed(dim)
+    L, H, F = 4, 3, 300
+    with ForcingKVCache(n_layers=L, n_heads=H, head_dim=dim, tokens_per_frame=F, frames_per_chunk=2, n_sink_frames=1,
+                        window_frames=6, n_segments=3, keep_budget_permille=700,
+                        head_is_static=np.zeros((L, H), np.uint8)) as cache:
+        def rand(n):
+            return torch.randn((n, H, dim), generator=g, device="cuda").to(torch.bfloat16)
+        for l in range(L):
+            cache.append_frames(l, rand(7 * F), rand(7 * F))
+            cache.set_current(l, rand(2 * F), rand(2 * F))
+        cache.compress()
+        q = [rand(2 * F) for _ in range(L)]
+        want = [cache.attend(l, q[l]) for l in range(L)]
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        for _ in range(20):
+            outs = [torch.empty_like(x) for x in q]
+            torch.cuda.synchronize()
+            for l in range(L):
+                cache.attend(l, q[l], outs[l], stream=streams[l % 2])
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(outs, want))
+        assert cache.sync_status() == 0
