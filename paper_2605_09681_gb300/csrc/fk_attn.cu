@@ -248,25 +248,6 @@ __device__ __forceinline__ void umma_commit(uint64_t* b) {
         "=r"(v[31])                                                                         \
       : "r"(taddr))
 
-#define FK_TMEM_LD64(taddr, v)                                                              \
-  asm volatile(                                                                             \
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"  \
-      "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33," \
-      "%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54," \
-      "%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];"                                        \
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),  \
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),           \
-        "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),        \
-        "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),        \
-        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),        \
-        "=r"(v[31]), "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]),        \
-        "=r"(v[37]), "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]), "=r"(v[42]),        \
-        "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]), "=r"(v[48]),        \
-        "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]),        \
-        "=r"(v[55]), "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]),        \
-        "=r"(v[61]), "=r"(v[62]), "=r"(v[63])                                               \
-      : "r"(taddr))
-
 #define FK_TMEM_ST32(taddr, v)                                                              \
   asm volatile(                                                                             \
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"   \
@@ -290,9 +271,6 @@ __device__ __forceinline__ void umma_commit(uint64_t* b) {
         "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]),      \
         "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory")
 
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
@@ -390,6 +368,19 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* s, float2 sc2, float2 
         pk[p] = pack_bf16(e[p].x, e[p].y);
       }
     }
+  }
+}
+
+// 32 logits -> the sums of exp2(s * sc + nm) in four chains
+__device__ __forceinline__ void exp_sum(const uint32_t* s, float2 sc2, float2 nm2, float2* ah) {
+  float2 e[16];
+#pragma unroll
+  for (int q = 0; q < 16 + kSkew; ++q) {
+    if (q < 16) {
+      const float2 x = ffma2(make_float2(__uint_as_float(s[2 * q]), __uint_as_float(s[2 * q + 1])), sc2, nm2);
+      e[q] = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+    }
+    if (q >= kSkew) ah[q & 3] = fadd2(ah[q & 3], e[q - kSkew]);
   }
 }
 
@@ -951,11 +942,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 // [generated | sink | other history | transition].  S = Q K^T runs on the tensor cores
 // (tcgen05, S double-buffered in 256 TMEM columns); no P V product is needed.  Per row the
 // softmax statistics are kept online (running max, total sum, and the three class sums,
-// rescaled together); the per-row fractions are summed per head in double.  A cluster of two
-// CTAs handles one (head, 128-row query tile), each CTA half of the key tiles (so the grid
-// fills the SMs in about three even waves instead of two, the second half empty); the
-// second CTA writes its row statistics into the first's shared memory (distributed shared
-// memory, one cluster barrier), and the first merges the two ranges.
+// rescaled together); the per-row fractions are summed per head in double.  A cluster of k >= 2
+// CTAs handles one (head, 128-row query tile), each CTA a k-th of the key tiles (two fill the SMs
+// in about three even waves at 480P instead of two, the second half empty; small windows take
+// more, see launch_head_profile); the other CTAs write their row statistics into the first's shared
+// memory (distributed shared memory, one cluster barrier), and the first merges the ranges.
+// What bounds it: the statistics warps (S waits for them; ~1000 cycles per key tile and SM sub-
+// partition where the exponentials alone take 512), not the MMAs (half of the time; D = 64 takes
+// nearly as long).  12 heads, 4680 queries, 34320 keys: 380 us (405 before the tile of two classes
+// lost its branches and the loads their waits); 8 heads, 534 queries, 1246 keys, D = 64: 12.2 us
+// (16.4 with two CTAs per query tile).  Tried: S released before the sums (registers for 128
+// columns), no faster; loads running ahead into the next tile, slower.
 //   warps 0-3  statistics of rows 0..127 (TMEM lanes), one thread per row;
 //   warp 4     TMA: the query tile once, key tiles into a two-stage ring;
 //   warp 5     tcgen05.mma: S_b = Q K_j^T for b = j mod 2, once the statistics warps have
@@ -971,12 +968,13 @@ struct ProfLayout {
   static constexpr int kOffQ = 0;
   static constexpr int kOffK = kOffQ + kQ;
   static constexpr int kOffBar = kOffK + 2 * kK;
-  static constexpr int kOffPart = kOffBar + 256;      // the cluster peer's row statistics
+  static constexpr int kOffPart = kOffBar + 256;      // row statistics of peer 1 of the cluster
   static constexpr int kSmem = kOffPart + kAttnBM * 8 * 4 + 1024;   // + alignment slack; two CTAs per SM
+  static_assert((kMaxKvSplits - 2) * kAttnBM * 8 * 4 <= 2 * kK, "statistics of peers 2.. over the key stages");
 };
 
 template <int D>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kProfThreads, 2)
+__global__ void __launch_bounds__(kProfThreads, 2)
 profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const ProfArgs a) {
   using Lay = ProfLayout<D>;
@@ -991,26 +989,38 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   // barrier use: q_full, k_full/k_empty (key ring), s_full[b] (S_b written), p_full[b]
   // (S_b read by the four statistics warps), fin
 
-  float* part = reinterpret_cast<float*>(smem + Lay::kOffPart);   // [row][8]: m l cg cs ct ok
+  // [row][8]: m l cg cs ct ok of CTA r >= 1 of the cluster; of the third CTA on over the key
+  // stages, once every CTA is done with them
+  auto part_of = [&](uint32_t r) {
+    return reinterpret_cast<float*>(r == 1 ? smem + Lay::kOffPart : sK + (r - 2) * (kAttnBM * 8 * 4));
+  };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = warp * 32 + lane;                 // query row of a statistics thread
-  // A cluster of two CTAs = one (head, query tile); CTA r of the cluster takes key tiles
-  // [j0, j0 + nt) of the head's window (r = 0 the first half, r = 1 the rest).
-  uint32_t rank;
+  // A cluster of k CTAs = one (head, query tile); CTA r of the cluster takes key tiles [j0, j0 + nt)
+  // of the head's window, the r-th of k even ranges.
+  uint32_t rank, k;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int pair = blockIdx.x >> 1;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(k));
+  const int pair = blockIdx.x / k;
   const int head = pair / a.n_qtiles;
   const int q0 = (pair - head * a.n_qtiles) * kAttnBM;
   const int nk = a.Nk;
   const int nt_all = (nk + kAttnBN - 1) / kAttnBN;
-  const int j0 = rank ? nt_all / 2 : 0;
-  const int nt = rank ? nt_all - nt_all / 2 : nt_all / 2;   // may be 0 (one key tile in all)
+  const int j0 = (int)((int64_t)nt_all * rank / k);
+  const int nt = (int)((int64_t)nt_all * (rank + 1) / k) - j0;   // may be 0 (fewer key tiles than CTAs)
   // row statistics of this CTA's keys (statistics warps): running max (log2 domain), total
   // sum and the class sums, all relative to m
   float m = -INFINITY, l = 0.0f, cg = 0.0f, cs = 0.0f, ct = 0.0f;
   bool ok = true;
 
-  if (threadIdx.x == 0) {
+  // the TMA warp makes the barriers and starts the first loads before the CTA meets
+  auto load_k = [&](int j) {                          // key tile j into its stage
+    const int st = j & 1;
+    mbar_expect_tx(&bar->k_full[st], Lay::kK);
+    for (int h = 0; h < kHalves; ++h)
+      tma_load_3d(sK + st * Lay::kK + h * 16384, &tmK, &bar->k_full[st], h * 64, head, (j0 + j) * kAttnBN);
+  };
+  if (warp == kWarpProfTma && lane == 0) {
     mbar_init(&bar->q_full, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bar->k_full[i], 1);
@@ -1021,7 +1031,12 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     mbar_init(&bar->fin, 1);
     bar->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_expect_tx(&bar->q_full, Lay::kQ);
+    for (int h = 0; h < kHalves; ++h)
+      tma_load_3d(sQ + h * 16384, &tmQ, &bar->q_full, h * 64, head, q0);
+    for (int j = 0; j < min(2, nt); ++j) load_k(j);
   }
+  __syncwarp();
   if (warp == kWarpProfMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(su32(&bar->tmem_base)), "r"(kTmemCols) : "memory");
@@ -1034,18 +1049,12 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
   if (warp == kWarpProfTma) {
     if (lane == 0) {
-      int lastK[2] = {-1, -1};
+      int lastK[2] = {nt > 0 ? 0 : -1, nt > 1 ? 0 : -1};
       bool ok = true;
-      mbar_expect_tx(&bar->q_full, Lay::kQ);
-      for (int h = 0; h < kHalves; ++h)
-        tma_load_3d(sQ + h * 16384, &tmQ, &bar->q_full, h * 64, head, q0);
-      for (int j = 0; j < nt; ++j) {
+      for (int j = 2; j < nt; ++j) {
         const int st = j & 1, u = j >> 1;
-        if (j >= 2 && !wait_phase(&bar->k_empty[st], (u - 1) & 1, bar, a.status)) { ok = false; break; }
-        mbar_expect_tx(&bar->k_full[st], Lay::kK);
-        for (int h = 0; h < kHalves; ++h)
-          tma_load_3d(sK + st * Lay::kK + h * 16384, &tmK, &bar->k_full[st], h * 64, head,
-                      (j0 + j) * kAttnBN);
+        if (!wait_phase(&bar->k_empty[st], (u - 1) & 1, bar, a.status)) { ok = false; break; }
+        load_k(j);
         lastK[st] = u;
       }
       if (!ok) {   // drain every load this thread issued before the CTA exits
@@ -1079,62 +1088,79 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     wait_phase(&bar->fin, 0, bar, a.status, false);
     __syncwarp();
   } else {
-    const int wq = warp;
-    const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
+    const uint32_t tRow = tmem + ((uint32_t)(warp * 32) << 16);
+    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
+    // key classes are contiguous ranges in the order generated, sink, other, transition
+    auto key_class = [&](int key) { return key < a.g_end ? 0 : key < a.s_end ? 1 : key >= a.t_begin ? 3 : 2; };
+    auto add = [&](int cls, float sum) {
+      l += sum;
+      if (cls == 0) cg += sum;
+      else if (cls == 1) cs += sum;
+      else if (cls == 3) ct += sum;
+    };
     for (int j = 0; j < nt; ++j) {
       const int st = j & 1;
       if (!warp_wait(&bar->s_full[st], (j >> 1) & 1, bar, a.status)) { ok = false; break; }
       tc_fence_after();
+      const uint32_t tS = tRow + (uint32_t)(st * kAttnBN);
+      auto release = [&] {                           // S has been read
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar->p_full[st]);
+      };
+      // A full tile of one key class after the first (every row then has a finite running max m):
+      // the exponentials with m straight away, the next 32 columns' load in flight.  The tile's sum bounds each term, so only a sum above
+      // 2^8 (some key more than 1 above m in log2 units) needs the general path, which does the
+      // tile again.
+      const int k0 = (j0 + j) * kAttnBN;
+      if (j > 0 && nk - k0 >= kAttnBN && key_class(k0) == key_class(k0 + kAttnBN - 1)) {   // CTA-uniform
+        const float2 nm2 = make_float2(-m, -m);
+        float2 a2[4];
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const int kb = (j0 + j) * kAttnBN + half * 64;   // first key of this half
-        const int valid = min(64, nk - kb);          // uniform over the CTA
-        uint32_t sv[64];
-        FK_TMEM_LD64(tmem + lane_base + (uint32_t)(st * kAttnBN + half * 64), sv);
-        tmem_wait_ld();
-        if (half == 1) {                             // S_b is in registers: release it
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bar->p_full[st]);
+        for (int i = 0; i < 4; ++i) a2[i] = make_float2(0.0f, 0.0f);
+        uint32_t va[32], vb[32];
+        FK_TMEM_LD32(tS, va);
+        FK_TMEM_WAIT_LD32(va);
+        FK_TMEM_LD32(tS + 32, vb);
+        exp_sum(va, sc2, nm2, a2);
+        FK_TMEM_WAIT_LD32(vb);
+        FK_TMEM_LD32(tS + 64, va);
+        exp_sum(vb, sc2, nm2, a2);
+        FK_TMEM_WAIT_LD32(va);
+        FK_TMEM_LD32(tS + 96, vb);
+        exp_sum(va, sc2, nm2, a2);
+        FK_TMEM_WAIT_LD32(vb);
+        exp_sum(vb, sc2, nm2, a2);
+        const float2 s2 = fadd2(fadd2(a2[0], a2[1]), fadd2(a2[2], a2[3]));
+        const float sum = s2.x + s2.y;
+        if (!__any_sync(0xffffffffu, sum > 256.0f)) {                    // warp-uniform
+          release();
+          add(key_class(k0), sum);
+          continue;
         }
+      }
+      // General path: 32 columns at a time, with a max pass; classes by selection (a branch per key
+      // took 12000 cycles for a tile of two classes)
+#pragma unroll 1
+      for (int c0 = 0; c0 < 4; ++c0) {
+        const int kb = k0 + c0 * 32;                 // first key of these columns
+        const int valid = min(32, nk - kb);          // uniform over the CTA
+        float sv[32];
+        {
+          uint32_t u[32];
+          FK_TMEM_LD32(tS + c0 * 32, u);
+          FK_TMEM_WAIT_LD32(u);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) sv[c] = c < valid ? __uint_as_float(u[c]) : -INFINITY;
+        }
+        if (c0 == 3) release();
         if (valid <= 0) continue;
-        // key classes are contiguous ranges in the order generated, sink, other, transition
-        const int last = kb + valid - 1;
-        const int cls_first = kb < a.g_end ? 0 : kb < a.s_end ? 1 : kb >= a.t_begin ? 3 : 2;
-        const int cls_last = last < a.g_end ? 0 : last < a.s_end ? 1 : last >= a.t_begin ? 3 : 2;
-        // A full half of one key class after the first half (every row then has a finite
-        // running max m): the exponentials with m straight away.  The half's sum bounds each
-        // term, so only a sum above 2^8 (possibly a key more than 8 above m in log2 units)
-        // needs the max pass and lazy rescale below, which then redoes the half.
-        if (valid == 64 && cls_first == cls_last && (j > 0 || half > 0)) {   // CTA-uniform
-          const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nm2 = make_float2(-m, -m);
-          float2 a2[4];
+        float mxa[4];                                // four independent max chains
 #pragma unroll
-          for (int i = 0; i < 4; ++i) a2[i] = make_float2(0.0f, 0.0f);
+        for (int i = 0; i < 4; ++i) mxa[i] = sv[i];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const float2 x = ffma2(make_float2(__uint_as_float(sv[2 * q]), __uint_as_float(sv[2 * q + 1])),
-                                   sc2, nm2);
-            a2[q & 3] = fadd2(a2[q & 3], make_float2(fast_exp2(x.x), fast_exp2(x.y)));
-          }
-          const float2 s2 = fadd2(fadd2(a2[0], a2[1]), fadd2(a2[2], a2[3]));
-          const float sum = s2.x + s2.y;
-          if (!__any_sync(0xffffffffu, sum > 256.0f)) {                  // warp-uniform
-            l += sum;
-            if (cls_first == 0) cg += sum;
-            else if (cls_first == 1) cs += sum;
-            else if (cls_first == 3) ct += sum;
-            continue;
-          }
-        }
-        float mxa[8];                                // eight independent max chains
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mxa[i] = -INFINITY;
-#pragma unroll
-        for (int c = 0; c < 64; ++c)
-          if (c < valid) mxa[c & 7] = fmaxf(mxa[c & 7], __uint_as_float(sv[c]));
-        const float mx = fmaxf(fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])),
-                               fmaxf(fmaxf(mxa[4], mxa[5]), fmaxf(mxa[6], mxa[7])));
+        for (int c = 4; c < 32; ++c) mxa[c & 3] = fmaxf(mxa[c & 3], sv[c]);
+        const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
         const float m_new = fmaxf(m, mx * a.scale_log2);
         if (__any_sync(0xffffffffu, m_new > m + kRescaleThreshold)) {   // warp-uniform
           const float alpha = fast_exp2(m - m_new);  // 0 when m = -inf
@@ -1144,35 +1170,38 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           ct *= alpha;
           m = m_new;
         }
+        float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          sv[c] = fast_exp2(fmaf(sv[c], a.scale_log2, -m));
+          sum[c & 3] += sv[c];
+        }
+        const float all = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+        const int cls_first = key_class(kb), cls_last = key_class(kb + valid - 1);
         if (cls_first == cls_last) {
-          float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-          for (int c = 0; c < 64; ++c)
-            if (c < valid) acc[c & 3] += fast_exp2(fmaf(__uint_as_float(sv[c]), a.scale_log2, -m));
-          const float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-          l += sum;
-          if (cls_first == 0) cg += sum;
-          else if (cls_first == 1) cs += sum;
-          else if (cls_first == 3) ct += sum;
+          add(cls_first, all);
         } else {
+          const int ng = a.g_end - kb, ns = a.s_end - kb, nt0 = a.t_begin - kb;
+          float pg[2] = {0.0f, 0.0f}, ps[2] = {0.0f, 0.0f}, pt[2] = {0.0f, 0.0f};
 #pragma unroll
-          for (int c = 0; c < 64; ++c) {
-            if (c < valid) {
-              const int key = kb + c;
-              const float e = fast_exp2(fmaf(__uint_as_float(sv[c]), a.scale_log2, -m));
-              l += e;
-              if (key < a.g_end) cg += e;
-              else if (key < a.s_end) cs += e;
-              else if (key >= a.t_begin) ct += e;
-            }
+          for (int c = 0; c < 32; ++c) {
+            pg[c & 1] = fmaf(c < ng ? 1.0f : 0.0f, sv[c], pg[c & 1]);
+            ps[c & 1] = fmaf(c >= ng && c < ns ? 1.0f : 0.0f, sv[c], ps[c & 1]);
+            pt[c & 1] = fmaf(c >= nt0 ? 1.0f : 0.0f, sv[c], pt[c & 1]);
           }
+          l += all;
+          cg += pg[0] + pg[1];
+          cs += ps[0] + ps[1];
+          ct += pt[0] + pt[1];
         }
       }
     }
-    if (rank == 1) {
-      // this CTA's row statistics go to the same row slot in the first CTA's shared memory
-      uint32_t dst;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(su32(part + row * 8)), "r"(0u));
+  }
+  if (k > 2) cluster_sync();
+  if (warp < kWarpProfTma) {
+    if (rank > 0) {
+      // this CTA's row statistics go to its slot of the same row in the first CTA's shared memory
+      const uint32_t dst = map_peer(su32(part_of(rank) + row * 8), 0);
       asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" :: "r"(dst), "f"(m), "f"(l),
                    "f"(cg), "f"(cs) : "memory");
       asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" :: "r"(dst + 16u), "f"(ct),
@@ -1187,20 +1216,23 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem),
                  "r"(kTmemCols) : "memory");
   }
-  // every thread of both CTAs: the second CTA's statistics have landed (release / acquire)
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // every thread of the cluster: the other CTAs' statistics have landed
+  cluster_sync();
   if (rank == 0 && warp < kWarpProfTma) {
-    // merge the two key ranges: with M = max(m0, m1), every sum s = s0 2^(m0 - M) + s1 2^(m1 - M)
-    const float* pp = part + row * 8;
-    const float pm = pp[0];
-    ok = ok && pp[5] != 0.0f;                       // warp-uniform: one warp of each CTA per row block
-    const float M = fmaxf(m, pm);
-    const float w0 = m == -INFINITY ? 0.0f : fast_exp2(m - M);
-    const float w1 = pm == -INFINITY ? 0.0f : fast_exp2(pm - M);
-    l = l * w0 + pp[1] * w1;
-    cg = cg * w0 + pp[2] * w1;
-    cs = cs * w0 + pp[3] * w1;
-    ct = ct * w0 + pp[4] * w1;
+    // merge the key ranges one by one: with M = max(m0, m1), every sum s = s0 2^(m0 - M) + s1 2^(m1 - M)
+    for (uint32_t r = 1; r < k; ++r) {
+      const float* pp = part_of(r) + row * 8;
+      const float pm = pp[0];
+      ok = ok && pp[5] != 0.0f;                     // warp-uniform: one warp of each CTA per row block
+      const float M = fmaxf(m, pm);
+      const float w0 = m == -INFINITY ? 0.0f : fast_exp2(m - M);
+      const float w1 = pm == -INFINITY ? 0.0f : fast_exp2(pm - M);
+      m = M;
+      l = l * w0 + pp[1] * w1;
+      cg = cg * w0 + pp[2] * w1;
+      cs = cs * w0 + pp[3] * w1;
+      ct = ct * w0 + pp[4] * w1;
+    }
     if (ok) {
       const bool in = q0 + row < a.Nq;
       float fg = in ? cg / l : 0.0f, fs = in ? cs / l : 0.0f, ft = in ? ct / l : 0.0f;
@@ -1227,20 +1259,33 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
 cudaError_t launch_head_profile(int head_dim, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                                 const ProfArgs& a, cudaStream_t s) {
-  const unsigned grid = (unsigned)(2 * a.n_qtiles * a.H);   // clusters of two CTAs
-  cudaError_t e;
-  if (head_dim == 128) {
-    e = cudaFuncSetAttribute(profile_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             ProfLayout<128>::kSmem);
-    if (e != cudaSuccess) return e;
-    profile_kernel<128><<<grid, kProfThreads, ProfLayout<128>::kSmem, s>>>(tmQ, tmK, a);
-  } else {
-    e = cudaFuncSetAttribute(profile_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             ProfLayout<64>::kSmem);
-    if (e != cudaSuccess) return e;
-    profile_kernel<64><<<grid, kProfThreads, ProfLayout<64>::kSmem, s>>>(tmQ, tmK, a);
-  }
-  return cudaGetLastError();
+  // Key ranges per (head, query tile): two, or more while the CTAs (two per SM) all run at once.
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (int64_t)a.n_qtiles * a.H;
+  const int key_tiles = (a.Nk + kAttnBN - 1) / kAttnBN;
+  int k = 2;
+  while (k < kMaxKvSplits && tiles * (k + 1) <= 2 * sms * 9 / 10 && k + 1 <= key_tiles) ++k;
+  void (*kern)(const CUtensorMap, const CUtensorMap, const ProfArgs) =
+      head_dim == 128 ? profile_kernel<128> : profile_kernel<64>;
+  const int smem = head_dim == 128 ? ProfLayout<128>::kSmem : ProfLayout<64>::kSmem;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(tiles * k));
+  cfg.blockDim = dim3(kProfThreads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)k;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, a);
 }
 
 cudaError_t attention_prepare(int head_dim) {

@@ -82,3 +82,29 @@ def test_key_splits_on_two_streams(dim):
             torch.cuda.synchronize()
             assert all(torch.equal(a, b) for a, b in zip(outs, want))
         assert cache.sync_status() == 0
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+@pytest.mark.parametrize("g,s,t,nk", [(300, 100, 90, 1000), (512, 0, 128, 1024), (33, 7, 1, 2090), (0, 0, 0, 700)])
+def test_profile_maximum_raised(dim, g, s, t, nk):
+    """Head profiling: keys that raise the running maximum in tiles of one class, of two classes and
+    in the last one, over 2 to 8 key ranges per query tile."""
+    import torch
+
+    import oracle as O
+    from fkharness import to_dev
+    from paper_2605_09681_gb300 import head_profile
+    rng = np.random.default_rng(nk + dim)
+    u = rng.choice([-1.0, 1.0], size=dim)
+    q = rng.standard_normal((200, 3, dim)) + 2.0 * u
+    for n in range(6):
+        k = rng.standard_normal((nk, 3, dim))
+        for pos, a in ((20, 0.25), (nk // 3, 0.5), (nk // 2, 1.0), (nk // 2 + 1, 1.5), (nk - 1, 2.0))[:n]:
+            k[pos] = a * u
+        qb, kb = W.to_bf16_bits(q), W.to_bf16_bits(k)
+        mass, status = head_profile(to_dev(qb), to_dev(kb), g, s, t)
+        torch.cuda.synchronize()
+        qf, kf = W.bf16_bits_to_f32(qb), W.bf16_bits_to_f32(kb)
+        ref = np.stack([O.head_attention_mass(qf[:, h], kf[:, h], g, s, t) for h in range(3)])
+        assert int(status.item()) == 0
+        assert np.abs(mass.cpu().numpy() - ref).max() <= 1e-4 * 200      # fp32 exponentials and sums
