@@ -393,47 +393,35 @@ fk_status push_history(fk_handle* h, int layer, const bf16* tokK, const bf16* to
   LayerState& ls = h->layers[layer];
   const int nh0 = ls.nh, nh1 = ls.nh + nf;
   const int lo1 = h->W > 0 ? std::max(h->S, nh1 - h->W) : h->S;   // window after the push
-  const int64_t frame_elems = (int64_t)h->F * h->D;
-  for (int i = 0; i < nf; ++i) {
-    const int f = nh0 + i;
-    const bool sink = f < h->S;
-    const bool in_window = sink || f >= lo1;        // frames overwritten within this push are skipped
-    const bool is_anchor = !sink && f == nh1 - 1;
-    if (!in_window) continue;
-    ScatterArgs pa{}, va{};
-    pa.srcK = tokK + (int64_t)i * h->F * h->H * h->D;
-    pa.srcV = tokV + (int64_t)i * h->F * h->H * h->D;
-    pa.rows = h->F;
-    pa.heads = h->H;
-    pa.head_dim = h->D;
-    va = pa;
-    bool any_p = false, any_v = false;
-    for (int hd = 0; hd < h->H; ++hd) {
-      const HeadBuf& hb = h->heads[layer * h->H + hd];
-      if (hb.retains) {
-        pa.dstK[hd] = hb.pageK + ring_slot(h, f) * frame_elems;
-        pa.dstV[hd] = hb.pageV + ring_slot(h, f) * frame_elems;
-        any_p = true;
-      }
-      // every view holds the sinks; every dynamic view (and, unless they drop it, every
-      // static view) holds the anchor
-      if (sink || (is_anchor && (!hb.is_static || !h->drop_anchor))) {
-        const int64_t row = h->CF + (int64_t)(sink ? f : h->S) * h->F;
-        va.dstK[hd] = hb.viewK + row * h->D;
-        va.dstV[hd] = hb.viewV + row * h->D;
-        if (h->fp8) va.dstK8[hd] = h->viewK8 + (hb.row_base + row) * h->D;
-        if (h->fp8pv) va.dstV8[hd] = h->viewV8 + (hb.row_base + row) * h->D;
-        any_v = true;
-      }
-    }
-    if (any_p) {
-      fk_status st = launch(h, s, FK_KERNEL_APPEND, [&] { launch_scatter(pa, s); });
-      if (st != FK_OK) return st;
-    }
-    if (any_v) {
-      fk_status st = launch(h, s, FK_KERNEL_APPEND, [&] { launch_scatter(va, s); });
-      if (st != FK_OK) return st;
-    }
+  PrefillArgs a{};
+  a.srcK = tokK;
+  a.srcV = tokV;
+  a.F = h->F;
+  a.heads = h->H;
+  a.head_dim = h->D;
+  a.f0 = nh0;
+  // sinks, then the frames still in the window after the push (older ones are overwritten within it)
+  a.n_sink = std::max(0, std::min(h->S, nh1) - nh0);
+  a.win0 = std::max(std::max(nh0, h->S), lo1);
+  a.n_frames = a.n_sink + std::max(0, nh1 - a.win0);
+  a.anchor = nh1 - 1 >= h->S ? nh1 - 1 : -1;
+  a.S = h->S;
+  a.cap_nonsink = h->cap_nonsink;
+  a.CF = h->CF;
+  a.static_anchor = h->drop_anchor ? 0 : 1;
+  for (int hd = 0; hd < h->H; ++hd) {
+    const HeadBuf& hb = h->heads[layer * h->H + hd];
+    a.pageK[hd] = hb.retains ? hb.pageK : nullptr;
+    a.pageV[hd] = hb.retains ? hb.pageV : nullptr;
+    a.viewK[hd] = hb.viewK;
+    a.viewV[hd] = hb.viewV;
+    a.viewK8[hd] = h->fp8 ? h->viewK8 + hb.row_base * h->D : nullptr;
+    a.viewV8[hd] = h->fp8pv ? h->viewV8 + hb.row_base * h->D : nullptr;
+    a.is_static[hd] = hb.is_static ? 1 : 0;
+  }
+  if (a.n_frames > 0) {
+    fk_status st = launch(h, s, FK_KERNEL_APPEND, [&] { launch_prefill(a, s); });
+    if (st != FK_OK) return st;
   }
   ls.nh = nh1;
   ls.dirty = true;

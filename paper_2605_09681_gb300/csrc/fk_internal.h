@@ -134,18 +134,24 @@ struct CurrentArgs {
 };
 void launch_current(const CurrentArgs& a, cudaStream_t s);
 
-struct ScatterArgs {            // token-major [rows][H][D] -> per-head row-major [rows][D]
-  const bf16* srcK;
+struct PrefillArgs {            // token-major [nf*F][H][D] -> page rings, sink and anchor slots
+  const bf16* srcK;             // frame f0 on
   const bf16* srcV;
-  int rows;
-  int heads;
-  int head_dim;
-  bf16* dstK[kMaxHeads];        // nullptr = skip this head
-  bf16* dstV[kMaxHeads];
-  uint8_t* dstK8[kMaxHeads];    // FP8 attention view rows: E4M3 copy of dstK (else nullptr)
-  uint8_t* dstV8[kMaxHeads];    // FP8 P V view rows: E4M3 copy of dstV (else nullptr)
+  int F, heads, head_dim;
+  int f0;                       // global number of the first source frame
+  int n_sink, win0, n_frames;   // frames f0 .. f0 + n_sink - 1 (sinks), then win0 .. ; n_frames in all
+  int anchor;                   // newest non-sink frame of the push, -1: none
+  int S, cap_nonsink, CF;
+  int static_anchor;            // 1: static views keep the anchor frame (Eq. 2)
+  bf16* pageK[kMaxHeads];       // page rings (nullptr: head keeps no history pages)
+  bf16* pageV[kMaxHeads];
+  bf16* viewK[kMaxHeads];
+  bf16* viewV[kMaxHeads];
+  uint8_t* viewK8[kMaxHeads];   // FP8 attention: E4M3 copies of the K views, same rows (else nullptr)
+  uint8_t* viewV8[kMaxHeads];   // FP8 P V: E4M3 copies of the V views (else nullptr)
+  unsigned char is_static[kMaxHeads];
 };
-void launch_scatter(const ScatterArgs& a, cudaStream_t s);
+void launch_prefill(const PrefillArgs& a, cudaStream_t s);
 
 // ------------------------------------------------------------------ scoring / selection
 struct ScoreItem {              // one (layer, head) whose keys are scored
