@@ -47,6 +47,13 @@ def _numel(x) -> int:
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the current device's current stream without building a Stream object: 0.6 us a call,
+            # torch.cuda.current_stream() 3.7
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                return torch.cuda.current_stream().cuda_stream
         if torch.cuda.is_available():
             return torch.cuda.current_stream().cuda_stream
         return None
@@ -67,6 +74,9 @@ def head_profile(Q, K, n_generate: int, n_sink: int, n_transition: int, mass=Non
     nk = K.shape[0]
     if tuple(K.shape[1:]) != (H, D):
         raise ValueError("Q and K disagree on heads / head_dim")
+    if mass is None and status is None:            # one zeroed buffer: one fill launch
+        buf = torch.zeros(H * 4 + 1, dtype=torch.float64, device=Q.device)
+        mass, status = buf[:H * 4].view(H, 4), buf[H * 4:].view(torch.int32)[:1]
     if mass is None:
         mass = torch.zeros((H, 4), dtype=torch.float64, device=Q.device)
     if status is None:
