@@ -400,7 +400,8 @@ __device__ __forceinline__ bool exceeds(const float2* ah, uint32_t ov) {
 // Rows [g0, g0 + rows) of the key splits' merge by one of 8 warps: with M = max_s m_s (log2 domain),
 // O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s as bf16, `stride` elements from row to row.  D / 4
 // lanes read a row, 16 bytes each; lane k first forms the S <= kS weights of the warp's k-th row.  A
-// load from a peer takes 600-900 cycles, so kRows row groups of every split are in flight.
+// load from a peer takes 600-900 cycles, so every split's (and kRows row groups') are in flight; more of
+// them cost more in instruction fetch than they hide (the code runs once per CTA).
 template <int D, int kS, int kRows>
 __device__ __forceinline__ void merge_rows(uint32_t part, uint32_t ml, int S, int g0, int rows, bf16* O, int stride,
                                            int warp, int lane) {
@@ -895,9 +896,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       cluster_sync();                               // every CTA's rows are in place
       const int rows = min(R, valid_rows - split * R);
       bf16* orow = a.O + ((int64_t)(q0 + split * R) * a.H + head) * D;
-      if (S <= 2) merge_rows<D, 2, 8>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
-      else if (S <= 4) merge_rows<D, 4, 4>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
-      else merge_rows<D, 8, 2>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      if (S <= 2) merge_rows<D, 2, 2>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      else if (S <= 4) merge_rows<D, 4, 1>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
+      else merge_rows<D, 8, 1>(su32(smem), su32(ml), S, split * R, rows, orow, a.H * D, warp, lane);
       cluster_sync();                               // every peer has read this CTA's rows
     } else if (ok) {
       // normalise, and through the warp's own 32 rows of shared memory (16-byte chunk c of row r at
