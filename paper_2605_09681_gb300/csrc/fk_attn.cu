@@ -953,19 +953,22 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 // in about three even waves at 480P instead of two, the second half empty; small windows take
 // more, see launch_head_profile); the other CTAs write their row statistics into the first's shared
 // memory (distributed shared memory, one cluster barrier), and the first merges the ranges.
-// What bounds it: the statistics warps (S waits for them; ~1000 cycles per key tile and SM sub-
-// partition where the exponentials alone take 512), not the MMAs (half of the time; D = 64 takes
-// nearly as long).  12 heads, 4680 queries, 34320 keys: 380 us (405 before the tile of two classes
-// lost its branches and the loads their waits); 8 heads, 534 queries, 1246 keys, D = 64: 12.2 us
-// (16.4 with two CTAs per query tile).  Tried: S released before the sums (registers for 128
-// columns), no faster; loads running ahead into the next tile, slower.
-//   warps 0-3  statistics of rows 0..127 (TMEM lanes), one thread per row;
-//   warp 4     TMA: the query tile once, key tiles into a two-stage ring;
-//   warp 5     tcgen05.mma: S_b = Q K_j^T for b = j mod 2, once the statistics warps have
-//              read S_b of tile j - 2 (they release it right after their TMEM loads).
-constexpr int kProfThreads = 192;
-constexpr int kWarpProfTma = 4;
-constexpr int kWarpProfMma = 5;
+// What bounds it: shared memory at D = 128 (a 128x128x16 MMA reads 8 KB in the 64 cycles it computes,
+// and the key tile is written besides: 768 cycles per tile where the MMAs take 512), the
+// exponentials at D = 64 (600 cycles per tile and SM sub-partition).  With one set of statistics
+// warps per CTA the two CTAs of an SM fell into step, computing and waiting at the same time.  12
+// heads, 4680 queries, 34320 keys: 372 us (405 with one set, its loads not overlapped and a branch
+// per key in tiles of two classes; D = 64 320, was 389); 8 heads, 534 queries, 1246 keys, D = 64:
+// 10.4 us (16.4 with two CTAs per query tile).  Tried: S released before the sums (registers for
+// 128 columns), no faster; loads running ahead into the next tile, slower.
+//   warps 0-7  statistics of rows 0..127 (TMEM lanes), one thread per row, warps 0-3 on the even key
+//              tiles, 4-7 on the odd ones (merged at the end);
+//   warp 8     TMA: the query tile once, key tiles into a two-stage ring;
+//   warp 9     tcgen05.mma: S_b = Q K_j^T for b = j mod 2, once the statistics warps have
+//              read S_b of tile j - 2.
+constexpr int kProfThreads = 320;
+constexpr int kWarpProfTma = 8;                    // warps 0-3 / 4-7: statistics of even / odd key tiles
+constexpr int kWarpProfMma = 9;
 
 template <int D>
 struct ProfLayout {
@@ -974,7 +977,8 @@ struct ProfLayout {
   static constexpr int kOffQ = 0;
   static constexpr int kOffK = kOffQ + kQ;
   static constexpr int kOffBar = kOffK + 2 * kK;
-  static constexpr int kOffPart = kOffBar + 256;      // row statistics of peer 1 of the cluster
+  static constexpr int kOffOdd = kOffBar + 256;       // row statistics of the odd key tiles
+  static constexpr int kOffPart = kOffOdd + kAttnBM * 8 * 4;   // row statistics of peer 1 of the cluster
   static constexpr int kSmem = kOffPart + kAttnBM * 8 * 4 + 1024;   // + alignment slack; two CTAs per SM
   static_assert((kMaxKvSplits - 2) * kAttnBM * 8 * 4 <= 2 * kK, "statistics of peers 2.. over the key stages");
 };
@@ -1001,7 +1005,8 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     return reinterpret_cast<float*>(r == 1 ? smem + Lay::kOffPart : sK + (r - 2) * (kAttnBM * 8 * 4));
   };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = warp * 32 + lane;                 // query row of a statistics thread
+  const int row = (warp & 3) * 32 + lane;           // query row of a statistics thread
+  const int grp = warp >> 2;                        // its key tiles: even (0) or odd (1)
   // A cluster of k CTAs = one (head, query tile); CTA r of the cluster takes key tiles [j0, j0 + nt)
   // of the head's window, the r-th of k even ranges.
   uint32_t rank, k;
@@ -1094,7 +1099,7 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     wait_phase(&bar->fin, 0, bar, a.status, false);
     __syncwarp();
   } else {
-    const uint32_t tRow = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t tS = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(grp * kAttnBN);
     const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
     // key classes are contiguous ranges in the order generated, sink, other, transition
     auto key_class = [&](int key) { return key < a.g_end ? 0 : key < a.s_end ? 1 : key >= a.t_begin ? 3 : 2; };
@@ -1104,22 +1109,20 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       else if (cls == 1) cs += sum;
       else if (cls == 3) ct += sum;
     };
-    for (int j = 0; j < nt; ++j) {
-      const int st = j & 1;
-      if (!warp_wait(&bar->s_full[st], (j >> 1) & 1, bar, a.status)) { ok = false; break; }
+    for (int j = grp; j < nt; j += 2) {              // S_j is in buffer j mod 2
+      if (!warp_wait(&bar->s_full[grp], (j >> 1) & 1, bar, a.status)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t tS = tRow + (uint32_t)(st * kAttnBN);
       auto release = [&] {                           // S has been read
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar->p_full[st]);
+        if (lane == 0) mbar_arrive(&bar->p_full[grp]);
       };
       // A full tile of one key class after the first (every row then has a finite running max m):
       // the exponentials with m straight away, the next 32 columns' load in flight.  The tile's sum bounds each term, so only a sum above
       // 2^8 (some key more than 1 above m in log2 units) needs the general path, which does the
       // tile again.
       const int k0 = (j0 + j) * kAttnBN;
-      if (j > 0 && nk - k0 >= kAttnBN && key_class(k0) == key_class(k0 + kAttnBN - 1)) {   // CTA-uniform
+      if (j > 1 && nk - k0 >= kAttnBN && key_class(k0) == key_class(k0 + kAttnBN - 1)) {   // CTA-uniform
         const float2 nm2 = make_float2(-m, -m);
         float2 a2[4];
 #pragma unroll
@@ -1203,8 +1206,31 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       }
     }
   }
+  // merge of a row's statistics with those of other keys: with M = max(m0, m1), every sum
+  // s = s0 2^(m0 - M) + s1 2^(m1 - M)
+  auto merge = [&](const float* pp) {
+    const float pm = pp[0];
+    ok = ok && pp[5] != 0.0f;                       // warp-uniform: one warp writes a row block
+    const float M = fmaxf(m, pm);
+    const float w0 = m == -INFINITY ? 0.0f : fast_exp2(m - M);
+    const float w1 = pm == -INFINITY ? 0.0f : fast_exp2(pm - M);
+    m = M;
+    l = l * w0 + pp[1] * w1;
+    cg = cg * w0 + pp[2] * w1;
+    cs = cs * w0 + pp[3] * w1;
+    ct = ct * w0 + pp[4] * w1;
+  };
+  if (warp < kWarpProfTma) {                        // the odd tiles' statistics to the even tiles' threads
+    float* odd = reinterpret_cast<float*>(smem + Lay::kOffOdd) + row * 8;
+    if (grp == 1) {
+      *reinterpret_cast<float4*>(odd) = make_float4(m, l, cg, cs);
+      *reinterpret_cast<float2*>(odd + 4) = make_float2(ct, ok ? 1.0f : 0.0f);
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (grp == 0) merge(odd);
+  }
   if (k > 2) cluster_sync();
-  if (warp < kWarpProfTma) {
+  if (warp < 4) {
     if (rank > 0) {
       // this CTA's row statistics go to its slot of the same row in the first CTA's shared memory
       const uint32_t dst = map_peer(su32(part_of(rank) + row * 8), 0);
@@ -1224,21 +1250,8 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   }
   // every thread of the cluster: the other CTAs' statistics have landed
   cluster_sync();
-  if (rank == 0 && warp < kWarpProfTma) {
-    // merge the key ranges one by one: with M = max(m0, m1), every sum s = s0 2^(m0 - M) + s1 2^(m1 - M)
-    for (uint32_t r = 1; r < k; ++r) {
-      const float* pp = part_of(r) + row * 8;
-      const float pm = pp[0];
-      ok = ok && pp[5] != 0.0f;                     // warp-uniform: one warp of each CTA per row block
-      const float M = fmaxf(m, pm);
-      const float w0 = m == -INFINITY ? 0.0f : fast_exp2(m - M);
-      const float w1 = pm == -INFINITY ? 0.0f : fast_exp2(pm - M);
-      m = M;
-      l = l * w0 + pp[1] * w1;
-      cg = cg * w0 + pp[2] * w1;
-      cs = cs * w0 + pp[3] * w1;
-      ct = ct * w0 + pp[4] * w1;
-    }
+  if (rank == 0 && warp < 4) {
+    for (uint32_t r = 1; r < k; ++r) merge(part_of(r) + row * 8);
     if (ok) {
       const bool in = q0 + row < a.Nq;
       float fg = in ? cg / l : 0.0f, fs = in ? cs / l : 0.0f, ft = in ? ct / l : 0.0f;
