@@ -103,9 +103,9 @@ enum {
  * only inexact step before the softmax.  fk_quantize_e4m3 applies the same rounding.
  * FP8: Q K^T as FP8_QK, and P V on E4M3 operands too, f32 accumulation: values are rounded to
  * E4M3 unscaled (elements within +-448), and each softmax numerator exp(l - m) is scaled by
- * 2^6 before its E4M3 rounding, m being the running row maximum, which lags the row maximum by
- * at most a factor 2 (so a numerator stays within 2^7); the row normaliser is the sum of the
- * unrounded scaled numerators.  Both FP8 precisions require head_dim 128. */
+ * 2^6 before its E4M3 rounding, m being an integer (in log2 units) running reference: the row
+ * maximum so far rounded up, lagging it by less than 2.76 (so a rounded numerator is at most 416);
+ * the row normaliser is the sum of the unrounded scaled numerators.  Both FP8 precisions require head_dim 128. */
 enum {
   FK_ATTN_BF16 = 0,
   FK_ATTN_FP8_QK = 1,

@@ -57,9 +57,10 @@ namespace {
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s per wait
 constexpr float kRescaleThreshold = 1.0f;          // log2 units: a part that exceeds the bound raises m
-// FP8 P V: P is stored as e4m3 of 2^6 exp2(s c - m), m an integer running reference (the
-// running max rounded up) that lags the row max by at most 2 (rescale threshold), so P stays
-// within 2^8 < 448; reference changes rescale O and l by exact powers of two
+// FP8 P V: P is stored as e4m3 of 2^6 exp2(s c - m), m an integer running reference (the running
+// max rounded up) that lags the row max by less than log2(432) - 6 = 2.76, so that a stored code is at
+// most 416 (a bound of 2^8 instead raised m, and rescaled O, so much more often that a launch took
+// 261 us and not 241); reference changes rescale O and l by exact powers of two
 constexpr float kRescaleThresholdFp8 = 2.0f;
 constexpr float kPShiftFp8 = 6.0f;
 
@@ -322,6 +323,15 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return d;
 }
 
+// four non-negative floats -> four E4M3 codes (lowest key in the low byte)
+__device__ __forceinline__ uint32_t e4m3x4(float2 a, float2 b) {
+  uint32_t w;
+  asm("{\n .reg .b16 lo, hi;\n cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n"
+      " cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n mov.b32 %0, {lo, hi};\n}"
+      : "=r"(w) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return w;
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&p);
@@ -364,8 +374,8 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* s, float2 sc2, float2 
       ah[p & 3] = fadd2(ah[p & 3], e[p]);
       if constexpr (kE4m3) {
         if (p & 1) {
-          pk[p >> 1] = e4m3x2(e[p - 1].x, e[p - 1].y) | (e4m3x2(e[p].x, e[p].y) << 16);
-          ov |= pk[p >> 1] + 0x07070707u;
+          pk[p >> 1] = e4m3x4(e[p - 1], e[p]);
+          ov |= pk[p >> 1] + 0x02020202u;
         }
       } else {
         pk[p] = pack_bf16(e[p].x, e[p].y);
@@ -387,9 +397,10 @@ __device__ __forceinline__ void exp_sum(const uint32_t* s, float2 sc2, float2 nm
   }
 }
 
-// Whether a numerator of these columns may exceed 2^8 in any lane (warp-uniform).  bf16: no more
-// than their sum does.  E4M3: exactly when a code is above 0x78; codes are non-negative and at
-// most 0x7E, so adding 7 to each byte sets its top bit then, without carries between bytes.
+// Whether a numerator of these columns may exceed the bound in any lane (warp-uniform).  bf16, 2^8: no more
+// than their sum does.  E4M3 (the bound is then 432, the values that round above 416 or saturate):
+// exactly when a code is 0x7E; codes are non-negative and at most 0x7E, so adding 2 to each byte sets
+// its top bit then, without carries between bytes.
 template <bool kE4m3>
 __device__ __forceinline__ bool exceeds(const float2* ah, uint32_t ov) {
   if constexpr (kE4m3) return __any_sync(0xffffffffu, (ov & 0x80808080u) != 0);
@@ -730,7 +741,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // P columns 16c..16c+15 come from S columns 32c..32c+31; FP8 P V: e4m3 codes of
       // 2^6 exp2(S*c - m), four per column, P columns 8c..8c+7): the A operand of PV.  On full
       // tiles after the first, P is computed with the running max m straight away, the next
-      // 32 columns' load in flight; a part whose numerators all stay within 2^8 is stored, else it
+      // 32 columns' load in flight; a part whose numerators all stay within the bound is stored, else it
       // is done again by general_part.
       // general_part(Chunks<c0, kN>): chunks c0 .. c0 + kN - 1 with a max pass, and m raised when it grows by
       // more than kThr (FP8 P V: m is the running max rounded up to an integer).  O_t holds PV of
@@ -788,13 +799,18 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             tc_fence_after();
           }
 #pragma unroll 1
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t o[32];
+          for (int c = 0; c < D / 32; c += 2) {
+            uint32_t o[32], o2[32];
             FK_TMEM_LD32(tO + c * 32, o);
+            FK_TMEM_LD32(tO + c * 32 + 32, o2);
             FK_TMEM_WAIT_LD32(o);
+            FK_TMEM_WAIT_LD32(o2);
 #pragma unroll
             for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
             FK_TMEM_ST32(tO + c * 32, o);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) o2[e] = __float_as_uint(__uint_as_float(o2[e]) * alpha);
+            FK_TMEM_ST32(tO + c * 32 + 32, o2);
           }
         }
         return true;
