@@ -762,6 +762,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // more than kThr (FP8 P V: m is the running max rounded up to an integer).  O_t holds PV of
       // every key before part c0: with part 0 PV_t(j-1) is complete (see MMA order), with part 1 the
       // keys of part 0 once pva_done says so.
+      // FP8 P V: tiles 1, 2, 4 .. 32 bring m up to date in every row.  m has little room before a
+      // numerator leaves E4M3, most rows outgrow it early, and a raise in any one of a tile's four warps
+      // delays the whole tile (480P launch 238 -> 228 us; twice as many such tiles 232)
+      const bool refresh = kFp8PV && j <= 32 && (j & (j - 1)) == 0;
       auto general_part = [&](auto chunks) -> bool {
         constexpr int c0 = decltype(chunks)::first, kN = decltype(chunks)::count;
         uint32_t sv[kN][32];
@@ -783,7 +787,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           for (int i = 0; i < 32; ++i) mxa[i & 3] = fmaxf(mxa[i & 3], __uint_as_float(sv[c][i]));
         const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
         const float m_new = fmaxf(m, kFp8PV ? ceilf(mx * sl2) : mx * sl2);
-        const bool raise = __any_sync(0xffffffffu, m_new > m + kThr);  // warp-uniform
+        const bool raise = __any_sync(0xffffffffu, m_new > m + (refresh && c0 == 0 ? 0.0f : kThr));   // warp-uniform
         float alpha = 1.0f;                          // 0 when m = -inf
         if (raise) {
           if constexpr (kFp8PV) {                    // integer references: an exact power of two
@@ -841,7 +845,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       uint32_t cb[32], ov = 0;
       float2 ah[4];
       bool general = true;
-      if (direct) {
+      if (direct && !refresh) {
         uint32_t ca[32], pk[3 * kW];
 #pragma unroll
         for (int i = 0; i < 4; ++i) ah[i] = make_float2(0.0f, 0.0f);
