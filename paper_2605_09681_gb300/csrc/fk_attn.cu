@@ -23,11 +23,11 @@
 //                      that no numerator exceeds that bound, else the part is done again with
 //                      a max pass that raises the running max and rescales O and the row sum.
 //                      What bounds it (clock64 timeline of one CTA, 12 heads x 25480 keys, D =
-//                      128): one key tile takes 2500 cycles for 2048 cycles of MMA; a tile's
-//                      softmax takes 1090 of them and its P waits ~500 for the tensor pipe.  One
+//                      128): one key tile takes ~2450 cycles for 2048 cycles of MMA; a tile's
+//                      softmax takes ~1090 of them and its P waits ~500 for the tensor pipe.  One
 //                      hand-over per tile, a vote and a store wait per 64 columns and S kept for
-//                      both took 1230; a denoising step then ran 321 us (now 304), a step under
-//                      FP8 Q K^T 326 us (now 290), a 1080P step 6.22 ms (now 5.61).  96 + 32:
+//                      both took 1230; a denoising step at 480P then ran 321 us (now 303), a step
+//                      under FP8 Q K^T 326 us (now 289), a 1080P step 6.22 ms (now 5.57).  96 + 32:
 //                      P V of the first part (384 cycles) covers the second's arithmetic (~190).
 // TMEM columns: S0 0-127, S1 128-255, O0 256.., O1 256+D.. (512 allocated).
 // FP8_QK variant (D = 128): the K tiles hold E4M3 codes (one 128-byte swizzle atom per row,
@@ -59,8 +59,8 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s per wait
 constexpr float kRescaleThreshold = 1.0f;          // log2 units: a part that exceeds the bound raises m
 // FP8 P V: P is stored as e4m3 of 2^6 exp2(s c - m), m an integer running reference (the running
 // max rounded up) that lags the row max by less than log2(432) - 6 = 2.76, so that a stored code is at
-// most 416 (a bound of 2^8 instead raised m, and rescaled O, so much more often that a launch took
-// 261 us and not 241); reference changes rescale O and l by exact powers of two
+// most 416 (with a bound of 2^8 m was raised, and O rescaled, so much more often that a 480P launch
+// took 261 us and not 241); reference changes rescale O and l by exact powers of two
 constexpr float kRescaleThresholdFp8 = 2.0f;
 constexpr float kPShiftFp8 = 6.0f;
 
@@ -487,9 +487,10 @@ __device__ __forceinline__ void merge_rows(uint32_t part, uint32_t ml, int S, in
 }
 
 // kSplit: a launch with key splits (kv_splits > 1): the splits of one pair of query tiles are the
-// CTAs of a cluster, merged at the end through distributed shared memory.  kFp8: Q K^T on E4M3 operands (D = 128).  kFp8PV (with kFp8): P V on
-// E4M3 operands too: V tiles from the E4M3 copy of the V view arena (one 128-byte swizzle atom
-// per key row), P written as e4m3 of 2^6 exp2(s c - m), four keys per TMEM column.
+// CTAs of a cluster, merged at the end through distributed shared memory.  kFp8: Q K^T on E4M3
+// operands (D = 128).  kFp8PV (with kFp8): P V on E4M3 operands too: V tiles from the E4M3 copy of
+// the V view arena (one 128-byte swizzle atom per key row), P written as e4m3 of 2^6 exp2(s c - m),
+// four keys per TMEM column.
 template <int D, bool kSplit, bool kFp8, bool kFp8PV = false>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -909,8 +910,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // Merge of the key splits: every CTA of the cluster leaves its 256 rows of unnormalised O (16-
       // byte chunk c of row g at chunk c ^ (g mod D/4): conflict-free) and their (m, l) in its shared
       // memory, and CTA r forms rows [r R, (r + 1) R) from all of them, reading whole rows of its
-      // peers.  Bound by the SM-to-SM network, ~13 B per cycle and SM: 128 KB take ~11000 cycles with
-      // 3 splits, as 16-byte stores to the owner took 17500.
+      // peers.  Bound by the SM-to-SM network, ~14 B per cycle and SM: 128 KB take ~9000 cycles with
+      // 3 splits (17500 as 16-byte stores to the owner).
       const int S = a.kv_splits, valid_rows = min(2 * kAttnBM, a.Nq - q0), R = (valid_rows + S - 1) / S;
       float2* ml = reinterpret_cast<float2*>(smem + 2 * kAttnBM * D * 4);
       if (ok) {
@@ -1153,9 +1154,9 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (lane == 0) mbar_arrive(&bar->p_full[grp]);
       };
       // A full tile of one key class after the first (every row then has a finite running max m):
-      // the exponentials with m straight away, the next 32 columns' load in flight.  The tile's sum bounds each term, so only a sum above
-      // 2^8 (some key more than 1 above m in log2 units) needs the general path, which does the
-      // tile again.
+      // the exponentials with m straight away, the next 32 columns' load in flight.  The tile's sum
+      // bounds each term, so only a sum above 2^8 (128 keys: some key at least 1 above m in log2
+      // units) needs the general path, which does the tile again.
       const int k0 = (j0 + j) * kAttnBN;
       if (j > 1 && nk - k0 >= kAttnBN && key_class(k0) == key_class(k0 + kAttnBN - 1)) {   // CTA-uniform
         const float2 nm2 = make_float2(-m, -m);

@@ -103,9 +103,10 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // takes ceil(tiles / k) tiles and a fixed cost (set-up, first loads, epilogue, and with k > 1 the
 // merge), on the `clusters[k]` clusters that the device holds at once.  Grids that leave SMs idle
 // (few heads or queries) or whose last wave is short are where splits pay.  Measured, k = 1 / best
-// (k chosen): 6 heads, 808 queries, 2828 and 2020 keys 38 / 21 us (5); 4 heads, 2412 queries,
-// 13132 and 4020 keys 135 / 48 us (4); 12 heads, 4680 queries, 15600 keys 328 / 293 us (2), 25480
-// and 7800 keys 286 us (1; 320 us with 2).  The overheads are fitted to such sweeps of k.
+// (k chosen): 6 heads, 808 queries, 2828 and 2020 keys 34 / 17 us (5); 4 heads, 2412 queries,
+// 13132 and 4020 keys 128 / 42 us (4); 12 heads, 4680 queries, 15600 keys 312 / 278 us (2), 25480
+// and 7800 keys 286 us (1; 320 us with 2).  The overheads are fitted to such sweeps of k: in one of
+// 15 shapes and k = 1..8 the count chosen was the fastest in each.
 int choose_kv_splits(const int* clusters, int n_qtiles, int H, const int* n_keys) {
   const double kOverheadTiles = 3.5, kMergeTiles = 2.5;
   int tiles[kMaxHeads], min_tiles = 1 << 30;
