@@ -989,14 +989,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 // in about three even waves at 480P instead of two, the second half empty; small windows take
 // more, see launch_head_profile); the other CTAs write their row statistics into the first's shared
 // memory (distributed shared memory, one cluster barrier), and the first merges the ranges.
-// What bounds it: shared memory at D = 128 (a 128x128x16 MMA reads 8 KB in the 64 cycles it computes,
-// and the key tile is written besides: 768 cycles per tile where the MMAs take 512), the
-// exponentials at D = 64 (600 cycles per tile and SM sub-partition).  With one set of statistics
-// warps per CTA the two CTAs of an SM fell into step, computing and waiting at the same time.  12
-// heads, 4680 queries, 34320 keys: 372 us (405 with one set, its loads not overlapped and a branch
-// per key in tiles of two classes; D = 64 320, was 389); 8 heads, 534 queries, 1246 keys, D = 64:
-// 10.4 us (16.4 with two CTAs per query tile).  Tried: S released before the sums (registers for
-// 128 columns), no faster; loads running ahead into the next tile, slower.
+// What bounds it: the statistics warps (the exponentials of a tile alone hold an SM sub-partition's
+// special-function unit for 512 cycles, as long as the MMAs take; each is active 63% of the time).
+// With one set of statistics warps per CTA the two CTAs of an SM fell into step, computing and
+// waiting at the same time.  12 heads, 4680 queries, 34320 keys: 372 us (405 with one set, its loads
+// not overlapped and a branch per key in tiles of two classes; D = 64 320, was 389); 8 heads, 534
+// queries, 1246 keys, D = 64: 10.4 us (16.4 with two CTAs per query tile).  Tried: S released before
+// the sums (registers for 128 columns), no faster; loads running ahead into the next tile, slower; the
+// query tile in tensor memory, which halves the operand fetch from shared memory (8 KB in the 64
+// cycles of a 128x128x16 MMA), no faster.
 //   warps 0-7  statistics of rows 0..127 (TMEM lanes), one thread per row, warps 0-3 on the even key
 //              tiles, 4-7 on the odd ones (merged at the end);
 //   warp 8     TMA: the query tile once, key tiles into a two-stage ring;
