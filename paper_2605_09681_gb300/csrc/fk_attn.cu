@@ -46,10 +46,7 @@
 // overlap the tail of the kernel before it in the stream (the compaction or current-chunk
 // kernel, which write the K/V views, or whatever kernel produced Q), and the TMA thread waits
 // for that kernel (griddepcontrol.wait) before its first load; every global write of this
-// kernel follows MMAs that consume those loads.  After that wait it lets the kernel that follows
-// start: a current-chunk kernel then takes the SMs as this launch drains, and waits for its end
-// before it touches anything; and since every CTA of this launch has seen the kernels before it
-// complete, the scoring kernel behind that one may read older frames without waiting.
+// kernel follows MMAs that consume those loads.  It never triggers its own dependents early.
 #include "fk_internal.h"
 
 namespace fk {
@@ -561,8 +558,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Q, K and V may have been written by the previous kernel of the stream
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // only now: a kernel that starts early may then rely on everything before this launch
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // bf16 query tiles: the MMA operand, or (FP8) the softmax threads' quantization input
     uint8_t* q_dst = kFp8 ? sQ16 : sQ;
     mbar_expect_tx(&bar->q_full, 2 * kQBytes);

@@ -61,11 +61,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 constexpr int kBatch = 2;
 template <int GPR>
 __global__ void __launch_bounds__(256, 4) current_kernel(const CurrentArgs a) {
-  pdl_wait();      // the views may still be read, the inputs written, by the kernel before
-  // the kernel that follows may start its prologue; it waits for this one.  Only now: a scoring
-  // kernel reads frames older than the chunk retired here without waiting, and an append before
-  // this one may have written them
-  pdl_trigger();
+  pdl_trigger();   // the kernel that follows may start its prologue; it waits for this one
   constexpr int TB = 256 / GPR;
   constexpr int D = GPR * 8;
   __shared__ int acc[(kFuseMaxFrames + 1) * TB * 4];   // [frame][segment][N hi, N lo, D hi, D lo]
@@ -365,18 +361,8 @@ void launch_current(const CurrentArgs& a, cudaStream_t s) {
   if (a.rows == 0 || a.heads == 0) return;
   const int gpr = a.head_dim / 8, tb = 256 / gpr;
   const dim3 grid((unsigned)((a.F + tb - 1) / tb), (unsigned)a.heads);
-  // programmatic launch: the CTAs take the SMs as an attention launch before them drains
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (gpr == 16) cudaLaunchKernelEx(&cfg, current_kernel<16>, a);
-  else cudaLaunchKernelEx(&cfg, current_kernel<8>, a);
+  if (gpr == 16) current_kernel<16><<<grid, 256, 0, s>>>(a);
+  else current_kernel<8><<<grid, 256, 0, s>>>(a);
 }
 
 void launch_prefill(const PrefillArgs& a, cudaStream_t s) {
