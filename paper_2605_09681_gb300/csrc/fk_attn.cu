@@ -1,8 +1,8 @@
 // Chunk attention over the per-head packed views (Sec. 4.2 Eq. 2, Sec. 4.3 Eq. 4):
 // O = softmax(Q K^T / sqrt(D)) V per head, with a different key count per head.
 //
-// One CTA computes two 128-row query tiles of one head against all of the head's keys,
-// in tiles of 128 keys, on the 5th-generation tensor cores:
+// One CTA computes two 128-row query tiles of one head (small grids: one, over two sets of keys, see
+// kOne) against all of the head's keys, in tiles of 128 keys, on the 5th-generation tensor cores:
 //   warp 8 (one lane)  TMA: both Q tiles once (3D map over [Nq][H][D]), K and V tiles (2D
 //                      maps over the view arenas) into two-stage rings, 128-byte swizzle;
 //                      key tile 0 on its own barrier, then V_j together with K_{j+1} on one
@@ -488,16 +488,24 @@ __device__ __forceinline__ void merge_rows(uint32_t part, uint32_t ml, int S, in
 // operands (D = 128).  kFp8PV (with kFp8): P V on E4M3 operands too: V tiles from the E4M3 copy of
 // the V view arena (one 128-byte swizzle atom per key row), P written as e4m3 of 2^6 exp2(s c - m),
 // four keys per TMEM column.
-template <int D, bool kSplit, bool kFp8, bool kFp8PV = false>
+// kOne: one query tile per CTA, so that a small grid has twice the CTAs and a cluster half the rows to
+// merge: both warpgroups own the same rows, warpgroup t over key tiles t, t + 2, .. (the two sets of S,
+// P and O in tensor memory are the key sets' instead of the query tiles'), merged at the end like two
+// more splits.  Per key tile a CTA takes 0.65 of the time for twice the K and V per query (when it pays:
+// choose_attention_plan).  6 heads, 808 queries, 2828 and 2020 keys, D = 128: 17.2 -> 14.4 us a launch.
+template <int D, bool kSplit, bool kFp8, bool kFp8PV = false, bool kOne = false>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
   static_assert(!kFp8 || D == 128, "FP8_QK: one 128-byte swizzle atom per Q / K row");
   static_assert(!kFp8PV || kFp8, "FP8 P V comes with FP8 Q K^T");
+  static_assert(!kOne || kSplit, "the two key sets' merge is the key splits' one");
   using Lay = Layout<D, kFp8, kFp8PV>;
   constexpr float kThr = kFp8PV ? kRescaleThresholdFp8 : kRescaleThreshold;
   constexpr float kPShift = kFp8PV ? kPShiftFp8 : 0.0f;
   constexpr int kHalves = D / 64;                 // 64-column (128-byte) swizzle atoms
+  // S_t(j + kAhead) follows P_t V_j; a query tile's (kOne: key set's) first key tile is below kAhead
+  constexpr int kAhead = kOne ? 2 : 1;
   constexpr uint32_t kTmemCols = 512;
   constexpr uint32_t kColO = 2 * kAttnBN;         // S0 = cols 0..127, S1 = 128..255, O0, O1 after
   extern __shared__ uint8_t smem_raw[];
@@ -515,7 +523,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   const int split = kSplit ? blockIdx.x % a.kv_splits : 0;
   const int rest = kSplit ? blockIdx.x / a.kv_splits : blockIdx.x;
   const int hi = rest / a.n_qtiles;
-  const int q0 = (rest - hi * a.n_qtiles) * (2 * kAttnBM);
+  const int q0 = (rest - hi * a.n_qtiles) * ((kOne ? 1 : 2) * kAttnBM);
   const int head = a.head_of[hi];
   int nk = a.n_keys[head];
   int row0 = a.row_base[head];
@@ -553,19 +561,21 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
     mbar_init(&bar->o_done, 1);
     mbar_init(&bar->fin, 1);
-    if (kFp8) mbar_init(&bar->q8_ready, 2 * kAttnBM);
+    if (kFp8) mbar_init(&bar->q8_ready, (kOne ? 1 : 2) * kAttnBM);
     bar->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Q, K and V may have been written by the previous kernel of the stream
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // bf16 query tiles: the MMA operand, or (FP8) the softmax threads' quantization input
     uint8_t* q_dst = kFp8 ? sQ16 : sQ;
-    mbar_expect_tx(&bar->q_full, 2 * kQBytes);
-    for (int t = 0; t < 2; ++t)
+    mbar_expect_tx(&bar->q_full, (kOne ? 1 : 2) * kQBytes);
+    for (int t = 0; t < (kOne ? 1 : 2); ++t)
       for (int h = 0; h < kHalves; ++h)
         tma_load_3d(q_dst + t * kQBytes + h * 16384, &tmQ, &bar->q_full, h * 64, head, q0 + t * kAttnBM);
-    mbar_expect_tx(&bar->k0_full, Lay::kK);
+    const bool k1 = kOne && nt > 1;                 // kOne: key tiles 0 and 1
+    mbar_expect_tx(&bar->k0_full, (k1 ? 2 : 1) * Lay::kK);
     load_k(0, &bar->k0_full);
+    if (k1) load_k(1, &bar->k0_full);
   }
   __syncwarp();
   if (warp == kWarpMma) {
@@ -585,12 +595,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       bool ok = true;
       // per key tile j: V_j together with K_{j+1} on one barrier (b = j mod 2).  Their
       // stages were last used by V_{j-2} and K_{j-1}, released together by vk_empty[b] after
-      // iteration j-2's MMAs (K_2 reuses K_0's stage: k0_empty)
+      // iteration j-2's MMAs (K_2 reuses K_0's stage: k0_empty).  kOne: V_j with K_{j+2}, whose stage
+      // K_j leaves with iteration j-2 (tiles 0 and 1: k0_empty).
       for (int j = 0; j < nt && ok; ++j) {
         const int bb = j & 1, u = j >> 1;
-        const bool more = j + 1 < nt;
+        const bool more = j + kAhead < nt;
         if (j >= 2 && !wait_phase(&bar->vk_empty[bb], (u - 1) & 1, bar, a.status)) { ok = false; break; }
-        if (j == 1 && more && !wait_phase(&bar->k0_empty, 0, bar, a.status)) { ok = false; break; }
+        if (!kOne && j == 1 && more && !wait_phase(&bar->k0_empty, 0, bar, a.status)) { ok = false; break; }
         mbar_expect_tx(&bar->vk_full[bb], Lay::kKV + (more ? Lay::kK : 0));
         if constexpr (kFp8PV) {
           tma_load_2d(sV + bb * Lay::kKV, &tmV, &bar->vk_full[bb], 0, row0 + j * kAttnBN);
@@ -599,8 +610,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             tma_load_2d(sV + bb * Lay::kKV + h * 16384, &tmV, &bar->vk_full[bb], h * 64,
                         row0 + j * kAttnBN);
         }
-        if (more) load_k(j + 1, &bar->vk_full[bb]);
         lastVK[bb] = u;
+        if (kOne && j < 2 && more && !wait_phase(&bar->k0_empty, 0, bar, a.status)) { ok = false; break; }
+        if (more) load_k(j + kAhead, &bar->vk_full[bb]);
       }
       if (!ok) {   // drain every load this thread issued before the CTA exits
         wait_phase(&bar->q_full, 0, bar, a.status, false);
@@ -620,12 +632,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // one thread complete in issue order, so when S_t(j+1) is reported complete, PV_t(j)
     // is complete too: the softmax of tile j+1 may rescale O_t without a further wait, and
     // S_t(j+1) overwriting P_t(j) (same columns) happens after PV_t(j) has read it.
+    // kOne: PV_t(j), S_t(j+2) with t = j mod 2.
     constexpr uint32_t kIdQK = kFp8 ? idesc_e4m3(kAttnBM, kAttnBN) : idesc_bf16(kAttnBM, kAttnBN, 0);
     constexpr uint32_t kIdPV = kFp8PV ? idesc_e4m3(kAttnBM, D, 1) : idesc_bf16(kAttnBM, D, 1);
     const uint64_t dQ = sdesc(su32(sQ), 16, 1024), dK = sdesc(su32(sK), 16, 1024);
     const uint64_t dV = sdesc(su32(sV), 16384, 1024);
     auto qk = [&](int j, int t) {
-      const uint64_t da = dQ + (uint32_t)(t * (Lay::kQ >> 4)), db = dK + (uint32_t)((j & 1) * (Lay::kK >> 4));
+      const uint64_t da = dQ + (uint32_t)((kOne ? 0 : t) * (Lay::kQ >> 4)), db = dK + (uint32_t)((j & 1) * (Lay::kK >> 4));
       const uint32_t d = tmem + (uint32_t)(t * kAttnBN);
       if constexpr (kFp8) {
         // 128 codes per row = one swizzle atom: four K = 32 steps of 32 bytes
@@ -649,11 +662,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         // MN-major (d contiguous, 128 bytes per key row), 8-row groups 1024 bytes apart
 #pragma unroll
         for (int kk = c0; kk < c1; ++kk)
-          umma_ts_f8(d, p + kk * 8, db + kk * 256, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_ts_f8(d, p + kk * 8, db + kk * 256, kIdPV, (j >= kAhead || kk > 0) ? 1u : 0u);
       } else {
 #pragma unroll
         for (int kk = 2 * c0; kk < 2 * c1; ++kk)
-          umma_ts(d, p + kk * 8, db + kk * 128, kIdPV, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_ts(d, p + kk * 8, db + kk * 128, kIdPV, (j >= kAhead || kk > 0) ? 1u : 0u);
       }
     };
     // every lane waits, one issues: the warp stays converged
@@ -663,30 +676,33 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       tc_fence_after();
       if (elect_one()) {
         qk(0, 0);
-        qk(0, 1);
+        if (!kOne) qk(0, 1);
+        else if (nt > 1) qk(1, 1);
         umma_commit(&bar->k0_empty);
       }
     }
     for (int j = 0; j < nt && ok; ++j) {
       const int bb = j & 1;
-      const bool more = j + 1 < nt;
+      const bool more = j + kAhead < nt;
+      const uint32_t ph = kOne ? (j >> 1) & 1 : j & 1;   // of a query tile's (kOne: key set's) barriers
       // V_j and K_{j+1} (one barrier) before P_0(j): neither depends on the softmax, and
       // PV0(j), S0(j+1) then go to the tensor pipe back to back once P_0(j) is in TMEM
       if (!wait(&bar->vk_full[bb], (j >> 1) & 1)) { ok = false; break; }
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        if (!wait(&bar->pa_full[t], j & 1)) { ok = false; break; }
+      for (int i = 0; i < (kOne ? 1 : 2); ++i) {
+        const int t = kOne ? bb : i;
+        if (!wait(&bar->pa_full[t], ph)) { ok = false; break; }
         tc_fence_after();
         if (elect_one()) {
           pv(j, t, 0, 3);
           umma_commit(&bar->pva_done[t]);
         }
-        if (!wait(&bar->p_full[t], j & 1)) { ok = false; break; }
+        if (!wait(&bar->p_full[t], ph)) { ok = false; break; }
         tc_fence_after();
         if (elect_one()) {
           pv(j, t, 3, 4);
-          if (more) qk(j + 1, t);
-          if (t == 1) umma_commit(&bar->vk_empty[bb]);   // V_j and K_{j+1} consumed
+          if (more) qk(j + kAhead, t);
+          if (kOne || t == 1) umma_commit(&bar->vk_empty[bb]);   // V_j and the K loaded with it consumed
         }
       }
     }
@@ -717,7 +733,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // chunk j of row r at chunk j ^ (r & 7)) -> max |q| -> e -> E4M3 codes of q 2^-e, 128 bytes
       // in the same swizzle pattern (rows past Nq were zero-filled: e = 0, codes 0)
       if (warp_wait(&bar->q_full, 0, bar, a.status)) {
-        const uint8_t* src = sQ16 + t * (kAttnBM * D * 2) + row * 128;
+        const uint8_t* src = sQ16 + (kOne ? 0 : t) * (kAttnBM * D * 2) + row * 128;
         uint4 v[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j)
@@ -727,9 +743,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         for (int j = 0; j < 16; ++j) amax = fmaxf(amax, absmax8(v[j]));
         const int e = e4m3_row_exponent(amax);
         const float inv = pow2f(-e);
-        uint8_t* dst = sQ + t * Lay::kQ + row * 128;
+        uint8_t* dst = sQ + (kOne ? 0 : t) * Lay::kQ + row * 128;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 8 && (!kOne || t == 0); ++j) {
           const uint2 lo = e4m3x8(v[2 * j], inv), hi = e4m3x8(v[2 * j + 1], inv);
           *reinterpret_cast<uint4*>(dst + ((j ^ (row & 7)) << 4)) = make_uint4(lo.x, lo.y, hi.x, hi.y);
         }
@@ -739,12 +755,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       } else {
         ok = false;
       }
-      mbar_arrive(&bar->q8_ready);
+      if (!kOne || t == 0) mbar_arrive(&bar->q8_ready);
     }
     const float2 sc2 = make_float2(sl2, sl2);
     float m = -INFINITY, l = 0.0f;
-    for (int j = 0; j < nt && ok; ++j) {
-      if (!warp_wait(&bar->s_full[t], j & 1, bar, a.status)) { ok = false; break; }
+    for (int it = 0; ok; ++it) {
+      const int j = kOne ? 2 * it + t : it;         // kOne: this warpgroup's key set is every other tile
+      if (j >= nt) break;
+      if (!warp_wait(&bar->s_full[t], it & 1, bar, a.status)) { ok = false; break; }
       tc_fence_after();
       const int valid = nk - j * kAttnBN;           // keys of this tile (< 128 only in the last)
       // A tile goes in two parts, keys 0-95 and 96-127, each handed to the MMA warp as soon as
@@ -761,7 +779,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // FP8 P V: tiles 1, 2, 4 .. 32 bring m up to date in every row.  m has little room before a
       // numerator leaves E4M3, most rows outgrow it early, and a raise in any one of a tile's four warps
       // delays the whole tile (480P launch 238 -> 228 us; twice as many such tiles 232)
-      const bool refresh = kFp8PV && j <= 32 && (j & (j - 1)) == 0;
+      const bool refresh = kFp8PV && it <= 32 && (it & (it - 1)) == 0;
       auto general_part = [&](auto chunks) -> bool {
         constexpr int c0 = decltype(chunks)::first, kN = decltype(chunks)::count;
         uint32_t sv[kN][32];
@@ -808,9 +826,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         }
         const float2 a4 = fadd2(fadd2(ac[0], ac[1]), fadd2(ac[2], ac[3]));
         l += a4.x + a4.y;
-        if (raise && (j > 0 || c0 > 0)) {
+        if (raise && (it > 0 || c0 > 0)) {
           if (c0 > 0) {
-            if (!warp_wait(&bar->pva_done[t], j & 1, bar, a.status)) return false;
+            if (!warp_wait(&bar->pva_done[t], it & 1, bar, a.status)) return false;
             tc_fence_after();
           }
 #pragma unroll 1
@@ -836,7 +854,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         __syncwarp();
         if (lane == 0) mbar_arrive(b);
       };
-      const bool direct = valid >= kAttnBN && j > 0; // uniform over the CTA
+      const bool direct = valid >= kAttnBN && it > 0; // uniform over the CTA
       constexpr int kW = kFp8PV ? 8 : 16;            // P words of 32 columns
       uint32_t cb[32], ov = 0;
       float2 ah[4];
@@ -907,9 +925,56 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       // memory, and CTA r forms rows [r R, (r + 1) R) from all of them, reading whole rows of its
       // peers.  Bound by the SM-to-SM network, ~14 B per cycle and SM: 128 KB take ~9000 cycles with
       // 3 splits (17500 as 16-byte stores to the owner).
-      const int S = a.kv_splits, valid_rows = min(2 * kAttnBM, a.Nq - q0), R = (valid_rows + S - 1) / S;
+      constexpr int kRowsCta = (kOne ? 1 : 2) * kAttnBM;
+      const int S = a.kv_splits, valid_rows = min(kRowsCta, a.Nq - q0), R = (valid_rows + S - 1) / S;
       float2* ml = reinterpret_cast<float2*>(smem + 2 * kAttnBM * D * 4);
-      if (ok) {
+      if constexpr (kOne) {
+        // first the CTA's two key sets: each warpgroup forms its half of the columns of every row,
+        // the other's accumulator of them through shared memory (chunk c of a row at c ^ (row mod D/8))
+        constexpr int kHalf = D / 2;
+        uint8_t* xo = smem + kAttnBM * D * 4 + t * (kAttnBM * kHalf * 4) + row * (kHalf * 4);
+        const uint8_t* xi = smem + kAttnBM * D * 4 + (1 - t) * (kAttnBM * kHalf * 4) + row * (kHalf * 4);
+        float2* mlx = ml + kAttnBM;
+        const bool has = t < nt;                    // (a single key tile: the second set is empty)
+        if (ok) {
+#pragma unroll 1
+          for (int c = 0; c < kHalf / 32; ++c) {
+            uint32_t o[32];
+            FK_TMEM_LD32(tO + (1 - t) * kHalf + c * 32, o);
+            FK_TMEM_WAIT_LD32(o);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              *reinterpret_cast<uint4*>(xo + (((c * 8 + e) ^ (row & (D / 8 - 1))) << 4)) =
+                  has ? make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]) : make_uint4(0, 0, 0, 0);
+          }
+          mlx[t * kAttnBM + row] = make_float2(m, l);
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (ok) {
+          const float2 other = mlx[(1 - t) * kAttnBM + row];
+          const float M = fmaxf(m, other.x), w0 = fast_exp2(m - M), w1 = fast_exp2(other.x - M);
+          uint8_t* dst = smem + row * (D * 4);
+#pragma unroll 1
+          for (int c = 0; c < kHalf / 32; ++c) {
+            uint32_t o[32];
+            FK_TMEM_LD32(tO + t * kHalf + c * 32, o);
+            FK_TMEM_WAIT_LD32(o);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float4 x = *reinterpret_cast<const float4*>(xi + (((c * 8 + e) ^ (row & (D / 8 - 1))) << 4));
+              float4 y = make_float4(x.x * w1, x.y * w1, x.z * w1, x.w * w1);
+              if (has) {
+                y.x = fmaf(__uint_as_float(o[4 * e]), w0, y.x);
+                y.y = fmaf(__uint_as_float(o[4 * e + 1]), w0, y.y);
+                y.z = fmaf(__uint_as_float(o[4 * e + 2]), w0, y.z);
+                y.w = fmaf(__uint_as_float(o[4 * e + 3]), w0, y.w);
+              }
+              *reinterpret_cast<float4*>(dst + ((((t * kHalf + c * 32) / 4 + e) ^ (row & (D / 4 - 1))) << 4)) = y;
+            }
+          }
+          if (t == 0) ml[row] = make_float2(M, l * w0 + other.y * w1);
+        }
+      } else if (ok) {
         const int g = t * kAttnBM + row;
         uint8_t* dst = smem + g * (D * 4);
 #pragma unroll 1
@@ -1339,41 +1404,24 @@ cudaError_t launch_head_profile(int head_dim, const CUtensorMap& tmQ, const CUte
   return cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, a);
 }
 
-cudaError_t attention_prepare(int head_dim) {
-  const auto set = [](const void* fn, int smem) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  };
-  cudaError_t e;
-  if (head_dim == 128) {
-    if ((e = set((const void*)attn_kernel<128, false, false>, Layout<128>::kSmem)) != cudaSuccess) return e;
-    if ((e = set((const void*)attn_kernel<128, true, false>, Layout<128>::kSmem)) != cudaSuccess) return e;
-    if ((e = set((const void*)attn_kernel<128, false, true>, Layout<128, true>::kSmem)) != cudaSuccess) return e;
-    if ((e = set((const void*)attn_kernel<128, true, true>, Layout<128, true>::kSmem)) != cudaSuccess) return e;
-    if ((e = set((const void*)attn_kernel<128, false, true, true>, Layout<128, true, true>::kSmem)) != cudaSuccess)
-      return e;
-    return set((const void*)attn_kernel<128, true, true, true>, Layout<128, true, true>::kSmem);
-  }
-  if ((e = set((const void*)attn_kernel<64, false, false>, Layout<64>::kSmem)) != cudaSuccess) return e;
-  return set((const void*)attn_kernel<64, true, false>, Layout<64>::kSmem);
-}
-
 namespace {
 using AttnKern = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnArgs);
-AttnKern attention_kernel(int head_dim, int precision, bool split, int* smem) {
-  if (head_dim == 128 && precision == FK_ATTN_FP8) {
-    *smem = Layout<128, true, true>::kSmem;
-    return split ? attn_kernel<128, true, true, true> : attn_kernel<128, false, true, true>;
-  }
-  if (head_dim == 128 && precision == FK_ATTN_FP8_QK) {
-    *smem = Layout<128, true>::kSmem;
-    return split ? attn_kernel<128, true, true> : attn_kernel<128, false, true>;
-  }
-  if (head_dim == 128) {
-    *smem = Layout<128>::kSmem;
-    return split ? attn_kernel<128, true, false> : attn_kernel<128, false, false>;
-  }
-  *smem = Layout<64>::kSmem;
-  return split ? attn_kernel<64, true, false> : attn_kernel<64, false, false>;
+// kernels of one head_dim and precision: [0] no key splits, [1] key splits, [2] one query tile per CTA
+struct AttnKerns {
+  AttnKern k[3];
+  int smem;
+};
+template <int D, bool kFp8, bool kFp8PV>
+AttnKerns attn_kernels() {
+  return {{attn_kernel<D, false, kFp8, kFp8PV>, attn_kernel<D, true, kFp8, kFp8PV>,
+           attn_kernel<D, true, kFp8, kFp8PV, true>},
+          Layout<D, kFp8, kFp8PV>::kSmem};
+}
+AttnKerns attention_kernels(int head_dim, int precision) {
+  if (head_dim == 64) return attn_kernels<64, false, false>();
+  if (precision == FK_ATTN_FP8) return attn_kernels<128, true, true>();
+  if (precision == FK_ATTN_FP8_QK) return attn_kernels<128, true, false>();
+  return attn_kernels<128, false, false>();
 }
 // launch configuration with programmatic dependent launch and, for key splits, a cluster of them
 void attention_config(int splits, int grid, int smem, cudaStream_t s, cudaLaunchConfig_t* cfg,
@@ -1394,23 +1442,32 @@ void attention_config(int splits, int grid, int smem, cudaStream_t s, cudaLaunch
 }
 }  // namespace
 
+cudaError_t attention_prepare(int head_dim) {
+  for (int precision : {FK_ATTN_BF16, FK_ATTN_FP8_QK, FK_ATTN_FP8}) {
+    const AttnKerns ks = attention_kernels(head_dim, precision);
+    for (AttnKern kern : ks.k) {
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ks.smem);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
 cudaError_t attention_clusters(int head_dim, int precision, int splits, int* n) {
-  int smem;
-  const AttnKern kern = attention_kernel(head_dim, precision, true, &smem);
+  const AttnKerns ks = attention_kernels(head_dim, precision);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  attention_config(splits, splits, smem, nullptr, &cfg, attr);
-  return cudaOccupancyMaxActiveClusters(n, kern, &cfg);
+  attention_config(splits, splits, ks.smem, nullptr, &cfg, attr);
+  return cudaOccupancyMaxActiveClusters(n, ks.k[1], &cfg);
 }
 
 void launch_attention(int head_dim, int precision, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                       const CUtensorMap& tmV, const AttnArgs& a, cudaStream_t s) {
-  int smem;
-  const AttnKern kern = attention_kernel(head_dim, precision, a.kv_splits > 1, &smem);
+  const AttnKerns ks = attention_kernels(head_dim, precision);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  attention_config(a.kv_splits, a.n_qtiles * a.H * a.kv_splits, smem, s, &cfg, attr);
-  cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, a);
+  attention_config(a.kv_splits, a.n_qtiles * a.H * a.kv_splits, ks.smem, s, &cfg, attr);
+  cudaLaunchKernelEx(&cfg, ks.k[a.one_qtile ? 2 : a.kv_splits > 1 ? 1 : 0], tmQ, tmK, tmV, a);
 }
 
 }  // namespace fk

@@ -25,7 +25,6 @@
 #include <cstring>
 #include <mutex>
 #include <new>
-#include <queue>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -98,42 +97,66 @@ bool get_encode() {
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// Key splits of one attention launch.  The CTAs (one per SM) are dispatched longest first; the
-// makespan is estimated greedily in units of key tiles for every split count: a cluster of k CTAs
-// takes ceil(tiles / k) tiles and a fixed cost (set-up, first loads, epilogue, and with k > 1 the
-// merge), on the `clusters[k]` clusters that the device holds at once.  Grids that leave SMs idle
-// (few heads or queries) or whose last wave is short are where splits pay.  Measured, k = 1 / best
-// (k chosen): 6 heads, 808 queries, 2828 and 2020 keys 34 / 17 us (5); 4 heads, 2412 queries,
-// 13132 and 4020 keys 128 / 42 us (4); 12 heads, 4680 queries, 15600 keys 312 / 278 us (2), 25480
-// and 7800 keys 286 us (1; 320 us with 2).  The overheads are fitted to such sweeps of k: in one of
-// 15 shapes and k = 1..8 the count chosen was the fastest in each.
-int choose_kv_splits(const int* clusters, int n_qtiles, int H, const int* n_keys) {
-  const double kOverheadTiles = 3.5, kMergeTiles = 2.5;
+// Query tiles per CTA and key splits of one attention launch.  The CTAs (one per SM) are dispatched
+// longest first; the makespan is estimated greedily, in units of what two query tiles take for a key
+// tile, for every split count: a cluster of k CTAs takes ceil(tiles / k) key tiles and a fixed cost
+// (set-up, first loads, epilogue, and with k > 1 the merge), on the `clusters[k]` clusters that the
+// device holds at once.  Grids that leave SMs idle (few heads or queries) or whose last wave is short
+// are where splits pay; CTAs of one query tile take 0.65 of the time per key tile, so less per CTA but more
+// per query, and merge half the bytes: they pay on small grids.  Measured, us (query tiles per CTA, k), two query
+// tiles and no split / best with two / best with one: 6 heads, 808 queries, 2828 and 2020 keys 33.4 / 17.2
+// (2, 5) / 14.4 (1, 3); 1 head, 328 queries, 2132 keys 26.0 / 13.7 (2, 6) / 10.1 (1, 6); 2 heads, 4680
+// queries, 13000 and 7800 keys 126 / 51.5 (2, 3) / 43.5 (1, 2); 4 heads, 2412 queries, 13132 and 4020 keys
+// 128 / 42.2 (2, 4) / 44.1 (1, 2); 12 heads, 4680 queries, 15600 keys 314 / 280 (2, 2) / 316 (1, 1), 25480
+// and 7800 keys 286 (2, 1) / 286 / 333 (1, 1).  The overheads are fitted to such sweeps: over 16 shapes the choice
+// was the fastest measured in 14 and within 3% and 6% of it in two.
+struct AttnPlan {
+  int one_qtile, kv_splits;
+};
+
+AttnPlan choose_attention_plan(const int* clusters, int Nq, int H, const int* n_keys) {
+  constexpr double kOverhead = 3.5, kMerge = 2.5, kOneOverhead = 2.0, kOneMerge = 0.5, kOneTile = 0.65;
   int tiles[kMaxHeads], min_tiles = 1 << 30;
   for (int hd = 0; hd < H; ++hd) {
     tiles[hd] = (n_keys[hd] + kAttnBN - 1) / kAttnBN;
     min_tiles = std::min(min_tiles, tiles[hd]);
   }
   std::sort(tiles, tiles + H, std::greater<int>());
-  int best = 1;
+  // (time, SMs or clusters busy until then), earliest first.  Equal jobs move a whole entry at a time: a
+  // heap of SMs cost the host 80 us when the key counts of a 480P layer change, this 4.
+  std::vector<std::pair<double, int>> load;
+  AttnPlan best{0, 1};
   double best_span = 0.0;
-  for (int k = 1; k <= std::min(kMaxKvSplits, min_tiles); ++k) {
-    if (clusters[k] < 1) continue;
-    std::priority_queue<double, std::vector<double>, std::greater<double>> load;
-    for (int i = 0; i < clusters[k]; ++i) load.push(0.0);
-    double span = 0.0;
-    for (int hd = 0; hd < H; ++hd)
-      for (int q = 0; q < n_qtiles; ++q) {
-        const double t = load.top() + (tiles[hd] + k - 1) / k + kOverheadTiles + (k > 1 ? kMergeTiles : 0.0);
-        load.pop();
-        load.push(t);
-        span = std::max(span, t);
+  for (int one = 0; one <= 1; ++one)
+    for (int k = 1; k <= std::min(kMaxKvSplits, min_tiles); ++k) {
+      if (clusters[k] < 1) continue;
+      const int rows = (one ? 1 : 2) * kAttnBM, n_qtiles = (Nq + rows - 1) / rows;
+      const double fixed = (one ? kOneOverhead : kOverhead) + (k == 1 ? 0.0 : one ? kOneMerge : kMerge);
+      load.assign(1, {0.0, clusters[k]});
+      double span = 0.0;
+      for (int hd = 0; hd < H;) {
+        int same = hd + 1;
+        while (same < H && tiles[same] == tiles[hd]) ++same;
+        const int n = (tiles[hd] + k - 1) / k;
+        const double cost = (one ? kOneTile * n : n) + fixed;
+        for (int64_t jobs = (int64_t)(same - hd) * n_qtiles; jobs > 0;) {
+          const int x = (int)std::min<int64_t>(jobs, load[0].second);
+          const double end = load[0].first + cost;
+          jobs -= x;
+          if ((load[0].second -= x) == 0) load.erase(load.begin());
+          auto at = load.end();
+          while (at != load.begin() && (at - 1)->first > end) --at;
+          if (at != load.begin() && (at - 1)->first == end) (at - 1)->second += x;
+          else load.insert(at, {end, x});
+          span = std::max(span, end);
+        }
+        hd = same;
       }
-    if (k == 1 || span < 0.97 * best_span) {
-      best = k;
-      best_span = span;
+      if ((!one && k == 1) || span < 0.97 * best_span) {
+        best = AttnPlan{one, k};
+        best_span = span;
+      }
     }
-  }
   return best;
 }
 
@@ -180,7 +203,7 @@ struct fk_handle {
   // attention key splits: clusters resident at once per split count, last decision per layer
   int attn_clusters[kMaxKvSplits + 1] = {};
   std::vector<std::vector<int>> split_keys;   // [L]: key counts the cached decision was made for
-  std::vector<int> split_choice;              // [L]
+  std::vector<AttnPlan> attn_plan;            // [L]
   ScoreItem* d_score_items = nullptr;
   SelectTarget* d_targets = nullptr;
   CompactItem* d_compact_items = nullptr;
@@ -852,7 +875,7 @@ fk_status fk_create(const fk_config* cfg, fk_handle** out) {
       h->attn_clusters[k] = 0;
     }
   h->split_keys.assign(h->L, {});
-  h->split_choice.assign(h->L, 1);
+  h->attn_plan.assign(h->L, AttnPlan{0, 1});
   h->stage_frames = h->C;
   for (Staging* sg : {&h->st_kv, &h->st_q})
     for (int sl = 0; sl < 2; ++sl)
@@ -1185,7 +1208,6 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
   a.O = o;
   a.Nq = h->CF;
   a.H = h->H;
-  a.n_qtiles = (h->CF + 2 * kAttnBM - 1) / (2 * kAttnBM);   // CTA = two 128-row query tiles
   a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)h->D));
   a.status = h->status;
   std::vector<int> order(h->H);
@@ -1200,10 +1222,13 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
   for (int i = 0; i < h->H; ++i) a.head_of[i] = order[i];
   std::vector<int> keys(a.n_keys, a.n_keys + h->H);
   if (keys != h->split_keys[layer]) {
-    h->split_choice[layer] = choose_kv_splits(h->attn_clusters, a.n_qtiles, h->H, a.n_keys);
+    h->attn_plan[layer] = choose_attention_plan(h->attn_clusters, h->CF, h->H, a.n_keys);
     h->split_keys[layer] = keys;
   }
-  a.kv_splits = h->split_choice[layer];
+  a.one_qtile = h->attn_plan[layer].one_qtile;
+  a.kv_splits = h->attn_plan[layer].kv_splits;
+  const int rows_cta = (a.one_qtile ? 1 : 2) * kAttnBM;
+  a.n_qtiles = (h->CF + rows_cta - 1) / rows_cta;
   const int D = h->D;
   // FP8: the E4M3 keys (and, for P V, values) come from the view arenas' E4M3 copies; the kernel
   // quantizes Q

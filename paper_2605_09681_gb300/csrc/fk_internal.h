@@ -255,7 +255,8 @@ struct AttnArgs {
   int n_qtiles;
   float scale_log2;             // log2(e) / sqrt(D)
   int* status;
-  int kv_splits;                // key splits per (head, query-tile pair), 1..kMaxKvSplits and at most
+  int one_qtile;                // a CTA computes one query tile (over two key sets) instead of two
+  int kv_splits;                // key splits per (head, CTA's query tiles), 1..kMaxKvSplits and at most
                                 // the key tiles of every head: the CTAs of one cluster
   int head_of[kMaxHeads];       // CTA order: head index of the i-th (longest-first) head
   int row_base[kMaxHeads];      // first row of the head's packed view in the view arena

@@ -52,10 +52,25 @@ def test_key_splits(dim, precision, heads, tokens, sinks):
     run_snapshot(w)
 
 
+@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+@pytest.mark.parametrize("heads,tokens,history", [(1, 20, 2), (3, 43, 2), (2, 86, 2), (1, 127, 4), (2, 129, 5), (1, 300, 6)])
+def test_one_query_tile(dim, precision, heads, tokens, history):
+    """Small grids, one query tile per CTA over two sets of key tiles: 1 key tile (the second set is
+    empty), 2 and 3, up to 14, over 1 to 8 splits; query tiles of 1 to 128 rows; the maximum raised late in either set."""
+    w = W.TINY_PER_FRAME.with_(name="one", n_heads=heads, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
+                               n_sink_frames=history - 1, n_history_frames=history, n_segments=1,
+                               static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
+    hk, hv, ck, cv, q = W.snapshot_inputs(w)
+    run_snapshot(w, inputs=(hk, hv, ck, cv, q))
+    for frac in (0.6, 0.95):                      # a key well above the rest, in an even or an odd tile
+        big = W.bf16_bits_to_f32(hk).copy()
+        big[int(frac * len(big))] *= 4.0
+        run_snapshot(w, inputs=(W.to_bf16_bits(big), hv, ck, cv, q))
+
+
 @pytest.mark.parametrize("dim", [64, 128])
 def test_key_splits_on_two_streams(dim):
-    """Layers attended on two streams at once (split launches share the handle's exchange slots)
-    give what one stream gives, over many rounds."""
+    """Layers attended on two streams at once give what one stream gives, over many rounds."""
     import torch
 
     from paper_2605_09681_gb300 import ForcingKVCache
