@@ -298,8 +298,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 // barrier over every thread of the cluster (release / acquire)
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 // shared-memory address of CTA `rank` of the cluster, and loads from such an address
 __device__ __forceinline__ uint32_t map_peer(uint32_t addr, int rank) {
@@ -1154,6 +1159,7 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  if (k == 2) cluster_arrive();                     // this CTA has started (waited for before the remote stores)
 
   if (warp == kWarpProfTma) {
     if (lane == 0) {
@@ -1326,7 +1332,11 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (grp == 0) merge(odd);
   }
-  if (k > 2) cluster_sync();
+  // Distributed shared memory may be written only once the owner has started, and the key stages (k > 2)
+  // only once it is done with them.  With two CTAs the barrier was arrived at when each began, so that
+  // neither waits here for the other's key range.
+  if (k == 2) cluster_wait();
+  else cluster_sync();
   if (warp < 4) {
     if (rank > 0) {
       // this CTA's row statistics go to its slot of the same row in the first CTA's shared memory

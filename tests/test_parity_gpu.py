@@ -354,6 +354,27 @@ def test_head_profile_sweep(i):
     _check_head_profile(q, k, g, s, t)
 
 
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("nk", [40, 128, 200])
+def test_head_profile_of_one_or_two_key_tiles_repeated(head_dim, nk):
+    """Two CTAs per query tile whose first has no key tile or one: the second hands its statistics over
+    as soon as it can, in launches queued behind one another."""
+    import torch
+
+    from paper_2605_09681_gb300 import head_profile
+    rng = np.random.default_rng(nk)
+    H, nq, g, s, t = 12, 1024, 20, 4, 7
+    qb, kb = (W.to_bf16_bits(rng.standard_normal((n, H, head_dim))) for n in (nq, nk))
+    Q, K = to_dev(qb), to_dev(kb)
+    out = [head_profile(Q, K, g, s, t) for _ in range(100)]
+    torch.cuda.synchronize()
+    qf, kf = W.bf16_bits_to_f32(qb), W.bf16_bits_to_f32(kb)
+    ref = np.stack([O.head_attention_mass(qf[:, h], kf[:, h], g, s, t) for h in range(H)])
+    for mass, status in out:
+        assert int(status.item()) == 0
+        assert np.abs(mass.cpu().numpy() - ref).max() <= 1e-4 * nq   # fp32 exponentials and sums
+
+
 def test_host_inputs_and_overlap_match_device_inputs():
     # the same stream driven with device tensors; with pageable host arrays (inputs copied
     # in call order, output copied back); and with pinned host tensors and host-input overlap
