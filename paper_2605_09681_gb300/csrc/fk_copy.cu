@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(256, 4) current_kernel(const CurrentArgs a) {
 constexpr int kPrefillBatch = 4;
 template <int GPR>
 __global__ void __launch_bounds__(256) prefill_kernel(const PrefillArgs a) {
-  // no early trigger: a scoring launch that follows reads older frames without waiting
+  // no early trigger: what usually follows is a current-chunk launch, an ordinary one
   constexpr int TB = 256 / GPR;
   constexpr int D = GPR * 8;
   const int h = blockIdx.y;

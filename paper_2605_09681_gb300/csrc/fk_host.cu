@@ -51,6 +51,7 @@ struct LayerState {
   int nh = 0;             // history frames appended
   bool has_current = false;
   bool dirty = false;     // appended since the last fk_compress
+  int fresh = 0;          // LayerRun::t_fresh of a scoring launch made now
   int scored_upto = 0;    // pairs (t, t+1) with t < scored_upto are scored
   int n_keep = 0;         // kept segments of each dynamic head (after fk_compress)
   int len_static = 0;     // keys of a static head
@@ -447,6 +448,7 @@ fk_status push_history(fk_handle* h, int layer, const bf16* tokK, const bf16* to
     fk_status st = launch(h, s, FK_KERNEL_APPEND, [&] { launch_prefill(a, s); });
     if (st != FK_OK) return st;
   }
+  ls.fresh = nh0;
   ls.nh = nh1;
   ls.dirty = true;
   if (ls.fuse_state == 1) ls.fuse_state = 2;   // frames the fused sums do not cover
@@ -536,6 +538,8 @@ fk_status update_current(fk_handle* h, int layer, bool retire, const void* K, co
   fk_status st = launch(h, s, FK_KERNEL_APPEND, [&] { launch_current(a, s); });
   if (st != FK_OK) return st;
   if (slot >= 0) FK_CUDA(cudaEventRecord(h->st_kv.freed[slot], s));
+  // a launch that retires nothing wrote no frame; the last chunk's stay behind the wait all the same
+  ls.fresh = retire ? ls.nh : std::max(ls.fresh, ls.nh - h->C);
   if (retire) {
     ls.nh += h->C;
     ls.dirty = true;
@@ -1055,14 +1059,13 @@ fk_status fk_compress(fk_handle* h, void* stream) {
       const int t_first = h->incremental ? std::max(r.t_lo, ls.scored_upto) : r.t_lo;
       const int last_t = r.t_lo + r.n_scoreable - 1;
       if (r.n_scoreable > 0 && t_first <= last_t) {
-        // the chunk the last append retired, [nh - C, nh), may still be in flight
         const int n_run = last_t + 2 - t_first;
         int n_read = n_run;
         if (ls.fuse_state == 1 && ls.fuse_t_first == t_first && ls.fuse_end == t_first + n_run)
           n_read = ls.fuse_n_read;   // the current-chunk kernel formed the rest of the sums
         else if (ls.fuse_state != 0)
           clear_sums = true;         // partial sums that match no run: clear, rescore all
-        sa.run[l] = {t_first, n_run, std::max(0, ls.nh - h->C), n_read};
+        sa.run[l] = {t_first, n_run, ls.fresh, n_read};
         any_run = true;
       } else if (ls.fuse_state != 0) {
         clear_sums = true;
@@ -1166,6 +1169,7 @@ fk_status fk_compress(fk_handle* h, void* stream) {
   }
   for (int l = 0; l < h->L; ++l) {
     LayerState& ls = h->layers[l];
+    ls.fresh = 0;         // the launches above are chained: none of them has waited for the others to end
     if (!ls.dirty) continue;
     ls.n_keep = keep_of[l];
     ls.dirty = false;

@@ -132,6 +132,7 @@ struct CurrentArgs {
   int* status;
   short score_target[kMaxHeads];   // sums target of head h, -1: not scored
 };
+// An ordinary launch (not a programmatic one): LayerRun::t_fresh relies on it.
 void launch_current(const CurrentArgs& a, cudaStream_t s);
 
 struct PrefillArgs {            // token-major [nf*F][H][D] -> page rings, sink and anchor slots
@@ -151,6 +152,7 @@ struct PrefillArgs {            // token-major [nf*F][H][D] -> page rings, sink 
   uint8_t* viewV8[kMaxHeads];   // FP8 P V: E4M3 copies of the V views (else nullptr)
   unsigned char is_static[kMaxHeads];
 };
+// An ordinary launch, as launch_current.
 void launch_prefill(const PrefillArgs& a, cudaStream_t s);
 
 // ------------------------------------------------------------------ scoring / selection
@@ -169,8 +171,14 @@ struct SelectTarget {           // one kept set: its layer and the score items f
 struct LayerRun {               // per layer: the run of frames t_first..t_first+n_run-1
   int t_first;
   int n_run;                    // frames whose sums the selection kernel finishes; 0 = none
-  int t_fresh;                  // frames >= t_fresh may come from the kernel launched just
-                                // before (the chunk it retired): read after its completion
+  // Frames >= t_fresh are read only after the scoring kernel's own wait, older ones (and the adds to
+  // the sums that follow from them) at once, while the launch before it still runs.  So whatever wrote an
+  // older frame, or read or cleared the sums, has to lie before an ordinary launch that itself lies before the
+  // scoring launch: an ordinary launch starts when everything before it has ended, a programmatic one does
+  // not (every kernel of the chain lets its successor start before it has waited itself).  t_fresh is
+  // therefore the first frame that the layer's newest current-chunk or prefill launch wrote, both ordinary, and
+  // 0 when the layer has had none since the last fk_compress.
+  int t_fresh;
   int n_read;                   // frames t_first.. the scoring kernel reads (the rest of the
                                 // run's sums were formed by the current-chunk kernel)
 };

@@ -378,8 +378,8 @@ __device__ __forceinline__ bool score_run(const ScoreArgs& a, int y, int j, int 
   const bf16* src0 = it.pagesK + (int64_t)tok0 * D;
   const int64_t frame_elems = (int64_t)a.F * D;
   auto issue = [&](int u) {
-    // frames the previous kernel of the stream wrote (the chunk it retired) are read only
-    // after that kernel has completed; older frames stream while it still runs
+    // frames that the kernel before may have written are read only after it has completed;
+    // older frames stream while it still runs (see LayerRun::t_fresh)
     if (!waited && run.t_first + k_load0 + u >= run.t_fresh) {
       pdl_wait();
       waited = true;
@@ -485,8 +485,8 @@ __device__ __forceinline__ bool score_run(const ScoreArgs& a, int y, int j, int 
 
 // Persistent grid: the frame-chunks of all scored items (item, segment, token chunk, frame)
 // form one flattened range split into equal contiguous pieces, one per CTA; a piece walks
-// its runs in order.  Launched with programmatic dependent launch after the current-chunk
-// kernel: a CTA streams frames older than the retired chunk while that kernel still runs,
+// its runs in order.  Launched with programmatic dependent launch, as a rule after the current-chunk
+// kernel: a CTA streams frames older than the retired chunk (run.t_fresh) while that kernel still runs,
 // waits for it (griddepcontrol.wait, thread 0, before its first fresh frame) and waits in
 // any case before it exits, so this grid completes only after that kernel, and the
 // selection and compaction chained behind it see the retired frames.
