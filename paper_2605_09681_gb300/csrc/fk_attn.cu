@@ -60,6 +60,10 @@ constexpr float kRescaleThreshold = 1.0f;          // log2 units: a part that ex
 // took 261 us and not 241); reference changes rescale O and l by exact powers of two
 constexpr float kRescaleThresholdFp8 = 2.0f;
 constexpr float kPShiftFp8 = 6.0f;
+// Running maximum (log2 domain) before any key.  Finite: keys whose logits are all -inf (products
+// below the float range) then give numerators exp2(-inf) = 0 and not exp2(-inf + inf) = NaN, also where
+// they fill all that one key split or key set begins with; the first finite logit raises it, with alpha = 0.
+constexpr float kNoMax = -3.402823466e38f;
 
 constexpr int kWarpTma = 8;                        // warps 0-3 / 4-7: softmax of query tile 0 / 1
 constexpr int kWarpMma = 9;
@@ -763,7 +767,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       if (!kOne || t == 0) mbar_arrive(&bar->q8_ready);
     }
     const float2 sc2 = make_float2(sl2, sl2);
-    float m = -INFINITY, l = 0.0f;
+    float m = kNoMax, l = 0.0f;
     for (int it = 0; ok; ++it) {
       const int j = kOne ? 2 * it + t : it;         // kOne: this warpgroup's key set is every other tile
       if (j >= nt) break;
@@ -807,11 +811,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
         const float m_new = fmaxf(m, kFp8PV ? ceilf(mx * sl2) : mx * sl2);
         const bool raise = __any_sync(0xffffffffu, m_new > m + (refresh && c0 == 0 ? 0.0f : kThr));   // warp-uniform
-        float alpha = 1.0f;                          // 0 when m = -inf
+        float alpha = 1.0f;                          // 0 when m = kNoMax
         if (raise) {
           if constexpr (kFp8PV) {                    // integer references: an exact power of two
             const float dm = m - m_new;
-            alpha = (m == -INFINITY || dm < -126.0f) ? 0.0f : pow2f((int)dm);
+            alpha = dm < -126.0f ? 0.0f : pow2f((int)dm);
           } else {
             alpha = fast_exp2(m - m_new);
           }
@@ -1123,7 +1127,7 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const int nt = (int)((int64_t)nt_all * (rank + 1) / k) - j0;   // may be 0 (fewer key tiles than CTAs)
   // row statistics of this CTA's keys (statistics warps): running max (log2 domain), total
   // sum and the class sums, all relative to m
-  float m = -INFINITY, l = 0.0f, cg = 0.0f, cs = 0.0f, ct = 0.0f;
+  float m = kNoMax, l = 0.0f, cg = 0.0f, cs = 0.0f, ct = 0.0f;
   bool ok = true;
 
   // the TMA warp makes the barriers and starts the first loads before the CTA meets
@@ -1275,7 +1279,7 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
         const float m_new = fmaxf(m, mx * a.scale_log2);
         if (__any_sync(0xffffffffu, m_new > m + kRescaleThreshold)) {   // warp-uniform
-          const float alpha = fast_exp2(m - m_new);  // 0 when m = -inf
+          const float alpha = fast_exp2(m - m_new);  // 0 when m = kNoMax
           l *= alpha;
           cg *= alpha;
           cs *= alpha;
@@ -1315,8 +1319,7 @@ profile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const float pm = pp[0];
     ok = ok && pp[5] != 0.0f;                       // warp-uniform: one warp writes a row block
     const float M = fmaxf(m, pm);
-    const float w0 = m == -INFINITY ? 0.0f : fast_exp2(m - M);
-    const float w1 = pm == -INFINITY ? 0.0f : fast_exp2(pm - M);
+    const float w0 = fast_exp2(m - M), w1 = fast_exp2(pm - M);   // 0 where no key had a finite logit
     m = M;
     l = l * w0 + pp[1] * w1;
     cg = cg * w0 + pp[2] * w1;
