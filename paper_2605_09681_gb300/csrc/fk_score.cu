@@ -126,11 +126,14 @@ __device__ __forceinline__ uint32_t rank_bits(float v) {
 // BottomK of one frame with many segments (token-level rules): the k-th smallest value by a radix
 // select (four passes of 256 bins over order-preserving bits), then the ids below it and, of its
 // ties, the lowest ids, written in ascending id order as frame-t segment ids into
-// out[0 .. min(k, bound)).  Block-uniform arguments, kSelectThreads = 256 threads.  A bitonic sort of
+// out[0 .. min(k, bound)).  Block-uniform arguments, kSelectThreads = 256 threads; `hist` is the
+// kSelectScratch bytes behind the staged values.  A bitonic sort of
 // (value, id) keys took log2(n)^2 / 2 barriers: 102 frames of 1560 random values 34 us, now 8.2.
+constexpr size_t kSelectScratch = (kSelectThreads + 2) * sizeof(int);
 __device__ void select_frame(const float* vals, int n, int k, int t, int* out, int bound, int* hist,
-                             int* warp_tot, int* base_off) {
+                             int* warp_tot) {
   static_assert(kSelectThreads == 256, "one thread per bin");
+  int* found = hist + kSelectThreads;            // the threshold's bin, and its rank within the bin
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint32_t prefix = 0, mask = 0;
   int remaining = min(k, n);                     // rank of the threshold among the values in prefix
@@ -154,13 +157,13 @@ __device__ void select_frame(const float* vals, int n, int k, int t, int* out, i
     __syncthreads();
     for (int w = 0; w < warp; ++w) inc += warp_tot[w];
     if (inc - cnt < remaining && remaining <= inc) {   // exactly one bin
-      base_off[0] = (int)threadIdx.x;
-      base_off[1] = remaining - (inc - cnt);
+      found[0] = (int)threadIdx.x;
+      found[1] = remaining - (inc - cnt);
     }
     __syncthreads();
-    prefix |= (uint32_t)base_off[0] << shift;
+    prefix |= (uint32_t)found[0] << shift;
     mask |= 255u << shift;
-    remaining = base_off[1];
+    remaining = found[1];
   }
   // `remaining` of the values equal to the threshold `prefix` are kept, the lowest ids
   int n_out = 0, n_tie = 0;                      // kept and ties so far (block-uniform)
@@ -185,7 +188,7 @@ __device__ void select_frame(const float* vals, int n, int k, int t, int* out, i
     n_out += (total & 0xFFFF) + min(remaining, n_tie + (total >> 16)) - min(remaining, n_tie);
     n_tie += total >> 16;
   }
-  __syncthreads();                               // hist, warp_tot and base_off may be used again
+  __syncthreads();                               // hist and warp_tot may be used again
 }
 
 // Selection kernel for a comparison rule with many segments per frame (per-frame scope): one
@@ -193,7 +196,7 @@ __device__ void select_frame(const float* vals, int n, int k, int t, int* out, i
 // independent.
 __global__ void __launch_bounds__(kSelectThreads) select_frames_kernel(const ScoreArgs a) {
   extern __shared__ float vals[];
-  __shared__ int hist[kSelectThreads], warp_tot[kSelectThreads / 32], base_off[2];
+  __shared__ int warp_tot[kSelectThreads / 32];
   const int tgi = blockIdx.x, f = blockIdx.y;
   const int l = a.targets[tgi].layer;
   pdl_trigger();
@@ -215,7 +218,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_frames_kernel(const Sco
     return;
   }
   __syncthreads();
-  select_frame(vals, n, k, t, out, bound, hist, warp_tot, base_off);
+  select_frame(vals, n, k, t, out, bound, reinterpret_cast<int*>(vals + n), warp_tot);
 }
 
 // Selection kernel: one CTA per selection target.  Finishes the pairs (t, t+1) scored by
@@ -224,7 +227,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_frames_kernel(const Sco
 // scores are staged in shared memory in candidate order (t - t_lo)*n + j.
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(const ScoreArgs a) {
   extern __shared__ float ssc[];
-  __shared__ int hist[kSelectThreads], warp_tot[kSelectThreads / 32], base_off[2];
+  __shared__ int warp_tot[kSelectThreads / 32];
+  __shared__ int base_off;
   const int tgi = blockIdx.x;
   const SelectTarget tg = a.targets[tgi];
   const int l = tg.layer;
@@ -279,12 +283,12 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const ScoreArgs 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (a.scope == FK_SCOPE_PER_FRAME && n > kRankDirect) {
     // many segments per frame (token-level rules): frame f's kept ids fill out[f k .. f k + k)
+    int* hist = reinterpret_cast<int*>(ssc + (int64_t)a.max_run * n);
     for (int f = 0; f < nT; ++f)
-      select_frame(ssc + f * n, n, a.k_frame, t_lo + f, out + f * a.k_frame, K - f * a.k_frame, hist, warp_tot,
-                   base_off);
+      select_frame(ssc + f * n, n, a.k_frame, t_lo + f, out + f * a.k_frame, K - f * a.k_frame, hist, warp_tot);
     return;
   }
-  if (threadIdx.x == 0) *base_off = 0;
+  if (threadIdx.x == 0) base_off = 0;
   __syncthreads();
   for (int b0 = 0; b0 < M; b0 += blockDim.x) {
     const int idx = b0 + threadIdx.x;
@@ -313,7 +317,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const ScoreArgs 
     const unsigned mask = __ballot_sync(0xffffffffu, keep);
     if (lane == 0) warp_tot[warp] = __popc(mask);
     __syncthreads();
-    int woff = *base_off;
+    int woff = base_off;
     for (int w = 0; w < warp; ++w) woff += warp_tot[w];
     const int pos = woff + __popc(mask & ((1u << lane) - 1u));
     if (keep && pos < K) out[pos] = t * n + j;   // bounded even if scores were not finite
@@ -321,7 +325,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const ScoreArgs 
     if (threadIdx.x == 0) {
       int tot = 0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += warp_tot[w];
-      *base_off += tot;
+      base_off += tot;
     }
     __syncthreads();
   }
@@ -537,17 +541,23 @@ constexpr size_t score_smem_bytes_d(int max_run) {
 size_t score_smem_bytes(int head_dim, int max_run) {
   return head_dim == 128 ? score_smem_bytes_d<128>(max_run) : score_smem_bytes_d<64>(max_run);
 }
-// The selection kernels stage `values` ranking values.  With many segments per frame the request
-// also has room for a sort of one frame (keys and flags), which the radix select does without: the
-// configurations that fit the shared memory limits stay the ones that always did.
+// The selection kernels stage `values` ranking values and, with many segments per frame, have the
+// radix select's scratch behind them.
 size_t select_smem_bytes(size_t values, int n_seg) {
-  size_t b = values * sizeof(float);
+  return values * sizeof(float) + (n_seg > kRankDirect ? kSelectScratch : 0);
+}
+// Whether a configuration's selection is accepted: what it took when a frame was sorted (keys and flags of
+// a power of two) has to fit beside the kernel's own shared memory.  What it takes now is never more, so this
+// is not a limit of the kernels: it keeps refused what was refused.
+bool select_fits(int max_run, int n_seg, size_t own, int optin) {
+  size_t b = (size_t)max_run * n_seg * sizeof(float);
   if (n_seg > kRankDirect) {
     size_t p = 1;
     while (p < (size_t)n_seg) p <<= 1;
     b = (b + 7) / 8 * 8 + p * 8 + (size_t)n_seg * 4;
   }
-  return b;
+  const int room = (int)b;
+  return room <= 48 * 1024 || (size_t)room + own <= (size_t)optin;
 }
 
 // launch with the programmatic-dependent-launch attribute: the kernel's prologue may
@@ -596,15 +606,18 @@ cudaError_t score_prepare(int head_dim, int max_run, int n_seg, int* max_ctas) {
   if (smem > 48 * 1024 && smem > fa.maxDynamicSharedSizeBytes)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int sel_smem = (int)select_smem_bytes((size_t)max_run * n_seg, n_seg);
-  if ((e = cudaFuncGetAttributes(&fa, (const void*)select_kernel)) != cudaSuccess) return e;
-  if (sel_smem > 48 * 1024 && sel_smem > fa.maxDynamicSharedSizeBytes)
-    e = cudaFuncSetAttribute((const void*)select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sel_smem);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
+  int dev = 0, sms = 0, optin = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  if ((e = cudaFuncGetAttributes(&fa, (const void*)select_kernel)) != cudaSuccess) return e;
+  if (!select_fits(max_run, n_seg, fa.sharedSizeBytes, optin)) return cudaErrorInvalidValue;
+  // the limit without a request is 48 KB less the kernel's own shared memory, so it is compared with, not 48 KB
+  // (select_frames_kernel stages one frame, and a frame that select_fits stays below it)
+  const size_t sel_smem = select_smem_bytes((size_t)max_run * n_seg, n_seg);
+  if (sel_smem > (size_t)fa.maxDynamicSharedSizeBytes && sel_smem + fa.sharedSizeBytes <= (size_t)optin)
+    e = cudaFuncSetAttribute((const void*)select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem);
+  if (e != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kScoreThreads, smem)) != cudaSuccess)
     return e;
   *max_ctas = sms * (per_sm > 0 ? per_sm : 1);
