@@ -94,7 +94,9 @@ struct Layout {
   static constexpr int kOffQ16 = kOffV + 2 * kKV; // FP8: two bf16 query tiles
   static constexpr int kOffBar = kOffQ16 + 2 * kQ16;
   static constexpr int kUsed = kOffBar + 256;
-  static_assert(2 * kAttnBM * (D * 4 + 8) <= kOffBar, "the key splits' rows of O and their (m, l)");
+  // the merge's rows of O (256, or 128 and the exchange of as many bytes), their (m, l) and, with one query
+  // tile per CTA, the two key sets' own
+  static_assert(2 * kAttnBM * D * 4 + 3 * kAttnBM * 8 <= kOffBar, "the merge leaves the barriers alone");
   // at least ~116 KB so that one CTA occupies an SM (its 512 TMEM columns are then free)
   static constexpr int kSmem = (kUsed + 1024) > 118 * 1024 ? (kUsed + 1024) : 118 * 1024;
 };
