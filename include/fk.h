@@ -264,6 +264,14 @@ FK_API fk_status fk_wait_outputs(fk_handle* h, void* stream);
  * `stream`.  FK_ERR_ARG for a null handle or a limit out of range. */
 FK_API fk_status fk_wait_selftest(fk_handle* h, int limit_us, void* stream);
 
+/* Attention launch plan, for tests and measurements (no counterpart in the paper): fk_attend of this
+ * handle computes `query_tiles` (1 or 2) 128-row query tiles per CTA over `kv_splits` (1..8) key
+ * splits instead of choosing both by the heads' key counts; 0 for both chooses again.  Results of
+ * two plans differ by rounding only.  FK_ERR_ARG for a null handle or values out of range;
+ * FK_ERR_CONFIG from fk_attend when a head has fewer 128-key tiles than splits, or the device
+ * cannot hold a cluster of that many CTAs. */
+FK_API fk_status fk_force_attention_plan(fk_handle* h, int query_tiles, int kv_splits);
+
 /* HBM calibration (no counterpart in the paper): reads `bytes` of device memory once with
  * 16-byte streaming loads from a grid of 8 CTAs per SM and does nothing else.  Timed with CUDA
  * events like the hot-path kernels, its duration is the practical floor for any single launch

@@ -274,6 +274,12 @@ class ForcingKVCache:
         FK_ERR_TIMEOUT."""
         _check(self._lib.fk_wait_selftest(self._h, int(limit_us), _stream(stream)), "fk_wait_selftest")
 
+    def force_attention_plan(self, query_tiles: int = 0, kv_splits: int = 0) -> None:
+        """Fix the attention's query tiles per CTA and key splits, for tests and measurements
+        (fk_force_attention_plan); 0, 0: chosen by the key counts."""
+        _check(self._lib.fk_force_attention_plan(self._h, int(query_tiles), int(kv_splits)),
+               "fk_force_attention_plan")
+
     def set_host_overlap(self, on: bool = True) -> None:
         """Overlap host transfers with queued work (see fk_set_host_overlap): host inputs must
         be final at call time; host outputs are complete after wait_outputs() (or

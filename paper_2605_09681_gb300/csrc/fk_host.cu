@@ -205,6 +205,7 @@ struct fk_handle {
   int attn_clusters[kMaxKvSplits + 1] = {};
   std::vector<std::vector<int>> split_keys;   // [L]: key counts the cached decision was made for
   std::vector<AttnPlan> attn_plan;            // [L]
+  AttnPlan forced_plan{0, 0};                 // fk_force_attention_plan (kv_splits 0: none)
   ScoreItem* d_score_items = nullptr;
   SelectTarget* d_targets = nullptr;
   CompactItem* d_compact_items = nullptr;
@@ -648,6 +649,14 @@ fk_status fk_wait_selftest(fk_handle* h, int limit_us, void* stream) {
                               static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? FK_OK
              : FK_ERR_CUDA;
+}
+
+fk_status fk_force_attention_plan(fk_handle* h, int query_tiles, int kv_splits) {
+  if (!h || query_tiles < 0 || query_tiles > 2 || kv_splits < 0 || kv_splits > kMaxKvSplits ||
+      (query_tiles == 0) != (kv_splits == 0))
+    return FK_ERR_ARG;
+  h->forced_plan = AttnPlan{query_tiles == 1 ? 1 : 0, kv_splits};
+  return FK_OK;
 }
 
 fk_status fk_set_host_overlap(fk_handle* h, int on) {
@@ -1184,6 +1193,13 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
   if (!Q || !O || !aligned16(Q) || !aligned16(O)) return FK_ERR_ARG;
   const LayerState& ls = h->layers[layer];
   if (!ls.has_current || ls.dirty) return FK_ERR_STATE;
+  if (const int k = h->forced_plan.kv_splits) {
+    for (int hd = 0; hd < h->H; ++hd) {
+      const int n = h->heads[layer * h->H + hd].is_static ? ls.len_static : ls.len_dynamic;
+      if (k > (n + kAttnBN - 1) / kAttnBN) return FK_ERR_CONFIG;
+    }
+    if (h->attn_clusters[k] < 1) return FK_ERR_CONFIG;
+  }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   FK_CUDA(cudaSetDevice(h->dev));
   const size_t bytes = (size_t)h->CF * h->H * h->D * 2;
@@ -1229,8 +1245,9 @@ fk_status fk_attend(fk_handle* h, int layer, const void* Q, void* O, void* strea
     h->attn_plan[layer] = choose_attention_plan(h->attn_clusters, h->CF, h->H, a.n_keys);
     h->split_keys[layer] = keys;
   }
-  a.one_qtile = h->attn_plan[layer].one_qtile;
-  a.kv_splits = h->attn_plan[layer].kv_splits;
+  const AttnPlan plan = h->forced_plan.kv_splits ? h->forced_plan : h->attn_plan[layer];
+  a.one_qtile = plan.one_qtile;
+  a.kv_splits = plan.kv_splits;
   const int rows_cta = (a.one_qtile ? 1 : 2) * kAttnBM;
   a.n_qtiles = (h->CF + rows_cta - 1) / rows_cta;
   const int D = h->D;

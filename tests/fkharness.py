@@ -74,14 +74,17 @@ def compare_layer(cache, orc, layer, Q_bits, O_dev, rows=None, heads=None, check
 
 
 def run_snapshot(w: W.Workload, rows=None, check_scores=True, inputs=None, head_map=None,
-                 full_heads=None, **cache_over):
+                 full_heads=None, plan=None, **cache_over):
     """Load a snapshot workload into the library and the oracle, compress, attend, compare
-    (`rows` of every head, then every row of the heads in `full_heads`)."""
+    (`rows` of every head, then every row of the heads in `full_heads`); `plan`: (query tiles per CTA,
+    key splits) of the attention instead of the library's choice."""
     import torch
     from paper_2605_09681_gb300 import ForcingKVCache
     hk, hv, ck, cv, q = inputs if inputs is not None else snapshot(w)
     hm = W.head_map(w) if head_map is None else head_map
     with ForcingKVCache.from_workload(w, hm, **cache_over) as cache:
+        if plan:
+            cache.force_attention_plan(*plan)
         cache.append_frames(0, to_dev(hk), to_dev(hv))
         cache.set_current(0, to_dev(ck), to_dev(cv))
         cache.compress()

@@ -24,9 +24,16 @@ def _spiked(w, spikes, seed):
     return b(K[F:]), b(V[F:]), b(K[:F]), b(V[:F]), b(q)
 
 
-@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+PRECISIONS = [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")]
+# (query tiles per CTA, key splits); None: the library's own choice
+PLANS = [(t, k) for t in (2, 1) for k in range(1, 9)]
+
+
+@pytest.mark.parametrize("dim,precision", PRECISIONS)
 @pytest.mark.parametrize("tokens", [384, 404, 418])       # last tile full, 60 keys, 102 keys
-def test_maximum_raised_in_either_part(dim, precision, tokens):
+@pytest.mark.parametrize("plan", [None, (2, 1), (1, 1), (2, 2)])
+def test_maximum_raised_in_either_part(dim, precision, tokens, plan):
+    """9 or 10 key tiles: all of them in one warpgroup's turn (2, 1), every other one (1, 1), half (2, 2)."""
     w = W.TINY_PER_FRAME.with_(name="parts", n_heads=2, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
                                n_sink_frames=1, n_history_frames=2, n_segments=2, static_heads=(0, 1),
                                attn_precision=precision)
@@ -37,35 +44,94 @@ def test_maximum_raised_in_either_part(dim, precision, tokens):
     spikes = [(100, 0.25), (128 + 40, 0.5), (256 + 120, 0.75), (512 + 3, 1.0), (512 + 127, 1.5),
               (last + 5, 2.0), (nk - 1, 2.5)]
     for n in range(len(spikes) + 1):           # the maximum stays at each of them once
-        run_snapshot(w, inputs=_spiked(w, spikes[:n], seed=n))
+        run_snapshot(w, inputs=_spiked(w, spikes[:n], seed=n), plan=plan)
 
 
-@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+@pytest.mark.parametrize("dim,precision", PRECISIONS)
+@pytest.mark.parametrize("plan", PLANS)
+def test_plans(dim, precision, plan):
+    """Every plan: one or two query tiles per CTA, 1 to 8 key splits, over 71 key tiles (each warpgroup gets
+    at least 4), the last one of 88 keys, with the maximum raised in early and late tiles of each range."""
+    F, frames = 312, 29                                      # 2 or 3 query tiles, 9048 keys
+    w = W.TINY_PER_FRAME.with_(name="plans", n_heads=2, head_dim=dim, tokens_per_frame=F, frames_per_chunk=1,
+                               n_sink_frames=frames - 2, n_history_frames=frames - 1, n_segments=1,
+                               static_heads=(0, 1), attn_precision=precision)
+    rng = np.random.default_rng(7)
+    nk, b = frames * F, W.to_bf16_bits
+    u = rng.choice([-1.0, 1.0], size=dim)
+    K, V = rng.standard_normal((nk, 2, dim)), rng.standard_normal((nk, 2, dim))
+    rise = np.linspace(0.1, 2.5, 24)                         # 24 keys, each above the ones before it
+    K[np.linspace(300, nk - 20, 24).astype(int)] = rise[:, None, None] * u
+    q = rng.standard_normal((F, 2, dim)) + 2.0 * u * (rng.random((F, 1, 1)) < 0.5)   # half of the rows follow u
+    rows = np.unique(np.r_[np.linspace(0, F - 1, 60).astype(int), 127, 128, 255, 256])
+    inputs = (b(K[F:]), b(V[F:]), b(K[:F]), b(V[:F]), b(q))
+    run_snapshot(w, rows=rows, inputs=inputs, plan=plan)
+
+
+@pytest.mark.parametrize("dim,precision", PRECISIONS)
+@pytest.mark.parametrize("heads,tokens,sinks", [(1, 341, 1), (1, 345, 1), (40, 225, 3)])
+@pytest.mark.parametrize("plan", PLANS)
+def test_plans_of_short_heads(dim, precision, heads, tokens, sinks, plan):
+    """8 or 9 key tiles, the last one of 127, 11 or 101 keys: ranges of one or two tiles, uneven over most splits,
+    key sets of one tile or none, query tiles of 89 to 256 rows."""
+    w = W.TINY_PER_FRAME.with_(name="short", n_heads=heads, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
+                               n_sink_frames=sinks, n_history_frames=sinks + 1, n_segments=1,
+                               static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
+    run_snapshot(w, rows=np.arange(0, tokens, 1 if heads == 1 else 9), plan=plan)
+
+
+def test_plans_that_do_not_fit():
+    """More splits than a head has key tiles are refused by the call, and the cache goes on as before."""
+    import torch
+
+    from fkharness import to_dev
+    from paper_2605_09681_gb300 import ForcingKVCache
+    from paper_2605_09681_gb300._lib import FkError
+    w = W.TINY_PER_FRAME.with_(name="fit", n_heads=1, tokens_per_frame=120, frames_per_chunk=1, n_sink_frames=1,
+                               n_history_frames=2, static_heads=(0,))
+    hk, hv, ck, cv, q = W.snapshot_inputs(w)
+    with ForcingKVCache.from_workload(w, W.head_map(w)) as cache:
+        cache.append_frames(0, to_dev(hk), to_dev(hv))
+        cache.set_current(0, to_dev(ck), to_dev(cv))
+        cache.compress()
+        want = cache.attend(0, to_dev(q))
+        for bad in ((3, 1), (0, 1), (1, 0), (2, 9), (-1, -1)):
+            with pytest.raises(FkError):
+                cache.force_attention_plan(*bad)
+        cache.force_attention_plan(2, 4)                     # 360 keys: three key tiles
+        with pytest.raises(FkError):
+            cache.attend(0, to_dev(q))
+        cache.force_attention_plan()
+        assert torch.equal(cache.attend(0, to_dev(q)), want)
+
+
+@pytest.mark.parametrize("dim,precision", PRECISIONS)
 @pytest.mark.parametrize("heads,tokens,sinks", [(1, 171, 1), (1, 256, 1), (1, 277, 1), (1, 341, 1), (2, 170, 1),
                                                 (40, 225, 3), (70, 225, 3), (1, 1040, 1)])
 def test_key_splits(dim, precision, heads, tokens, sinks):
-    """Grids whose heads have 4 to 9 (and 25) key tiles, the last one of 1 to 128 keys: 2 to 8 key
-    splits with uneven ranges, query tiles of 1 to 256 rows."""
+    """Grids whose heads have 4 to 9 (and 25) key tiles, the last one of 1 to 128 keys, as the library splits them
+    (one query tile per CTA, up to 8 splits)."""
     w = W.TINY_PER_FRAME.with_(name="splits", n_heads=heads, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
                                n_sink_frames=sinks, n_history_frames=sinks + 1, n_segments=1,
                                static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
     run_snapshot(w)
 
 
-@pytest.mark.parametrize("dim,precision", [(64, "bf16"), (128, "bf16"), (128, "fp8_qk"), (128, "fp8")])
+@pytest.mark.parametrize("dim,precision", PRECISIONS)
 @pytest.mark.parametrize("heads,tokens,history", [(1, 20, 2), (3, 43, 2), (2, 86, 2), (1, 127, 4), (2, 129, 5), (1, 300, 6)])
 def test_one_query_tile(dim, precision, heads, tokens, history):
     """Small grids, one query tile per CTA over two sets of key tiles: 1 key tile (the second set is
-    empty), 2 and 3, up to 14, over 1 to 8 splits; query tiles of 1 to 128 rows; the maximum raised late in either set."""
+    empty), 2 and 3, up to 17; query tiles of 1 to 128 rows; a larger key late in either set."""
     w = W.TINY_PER_FRAME.with_(name="one", n_heads=heads, head_dim=dim, tokens_per_frame=tokens, frames_per_chunk=1,
                                n_sink_frames=history - 1, n_history_frames=history, n_segments=1,
                                static_heads=tuple(range(heads)), attn_precision=precision, seed=heads + tokens)
     hk, hv, ck, cv, q = W.snapshot_inputs(w)
-    run_snapshot(w, inputs=(hk, hv, ck, cv, q))
-    for frac in (0.6, 0.95):                      # a key well above the rest, in an even or an odd tile
-        big = W.bf16_bits_to_f32(hk).copy()
-        big[int(frac * len(big))] *= 4.0
-        run_snapshot(w, inputs=(W.to_bf16_bits(big), hv, ck, cv, q))
+    for plan in (None, (1, 1)):
+        run_snapshot(w, inputs=(hk, hv, ck, cv, q), plan=plan)
+        for frac in (0.6, 0.95):                  # a key well above the rest, in an even or an odd tile
+            big = W.bf16_bits_to_f32(hk).copy()
+            big[int(frac * len(big))] *= 4.0
+            run_snapshot(w, inputs=(W.to_bf16_bits(big), hv, ck, cv, q), plan=plan)
 
 
 @pytest.mark.parametrize("dim", [64, 128])
@@ -100,10 +166,12 @@ def test_key_splits_on_two_streams(dim):
 
 
 @pytest.mark.parametrize("dim", [64, 128])
-@pytest.mark.parametrize("g,s,t,nk", [(300, 100, 90, 1000), (512, 0, 128, 1024), (33, 7, 1, 2090), (0, 0, 0, 700)])
-def test_profile_maximum_raised(dim, g, s, t, nk):
+@pytest.mark.parametrize("g,s,t,nk", [(300, 100, 90, 1000), (512, 0, 128, 1024), (33, 7, 1, 2090), (0, 0, 480, 700)])
+@pytest.mark.parametrize("heads,queries", [(3, 200), (8, 1000), (12, 1000)])
+def test_profile_maximum_raised(dim, g, s, t, nk, heads, queries):
     """Head profiling: keys that raise the running maximum in tiles of one class, of two classes and
-    in the last one, over 2 to 8 key ranges per query tile."""
+    in the last one; 6 or 8 key ranges per query tile of 1 to 3 tiles each (3 heads), 4 ranges of 1 to 5 (8), and
+    2 of 3 to 9 (12), where both sets of statistics warps get tiles after their first."""
     import torch
 
     import oracle as O
@@ -111,15 +179,16 @@ def test_profile_maximum_raised(dim, g, s, t, nk):
     from paper_2605_09681_gb300 import head_profile
     rng = np.random.default_rng(nk + dim)
     u = rng.choice([-1.0, 1.0], size=dim)
-    q = rng.standard_normal((200, 3, dim)) + 2.0 * u
+    q = rng.standard_normal((queries, heads, dim)) + 2.0 * u
     for n in range(6):
-        k = rng.standard_normal((nk, 3, dim))
+        k = rng.standard_normal((nk, heads, dim))
         for pos, a in ((20, 0.25), (nk // 3, 0.5), (nk // 2, 1.0), (nk // 2 + 1, 1.5), (nk - 1, 2.0))[:n]:
             k[pos] = a * u
         qb, kb = W.to_bf16_bits(q), W.to_bf16_bits(k)
         mass, status = head_profile(to_dev(qb), to_dev(kb), g, s, t)
         torch.cuda.synchronize()
         qf, kf = W.bf16_bits_to_f32(qb), W.bf16_bits_to_f32(kb)
-        ref = np.stack([O.head_attention_mass(qf[:, h], kf[:, h], g, s, t) for h in range(3)])
+        check = sorted({0, heads // 2, heads - 1})
+        ref = np.stack([O.head_attention_mass(qf[:, h], kf[:, h], g, s, t) for h in check])
         assert int(status.item()) == 0
-        assert np.abs(mass.cpu().numpy() - ref).max() <= 1e-4 * 200      # fp32 exponentials and sums
+        assert np.abs(mass.cpu().numpy()[check] - ref).max() <= 1e-4 * queries      # fp32 exponentials and sums
