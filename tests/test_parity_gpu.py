@@ -318,6 +318,7 @@ def _check_head_profile(q, k, g, s, t):
     torch.cuda.synchronize()
     got = mass.cpu().numpy()
     assert int(status.item()) == 0
+    assert mass.untyped_storage().nbytes() == H * 4 * 8 and status.untyped_storage().nbytes() == 4   # their own
     Qf, Kf = W.bf16_bits_to_f32(q), W.bf16_bits_to_f32(k)
     ref = np.stack([O.head_attention_mass(Qf[:, h], Kf[:, h], g, s, t) for h in range(H)])
     nq = q.shape[0]
