@@ -26,9 +26,10 @@
 //                      128): one key tile takes ~2450 cycles for 2048 cycles of MMA; a tile's
 //                      softmax takes ~1090 of them and its P waits ~500 for the tensor pipe.  One
 //                      hand-over per tile, a vote and a store wait per 64 columns and S kept for
-//                      both took 1230; a denoising step at 480P then ran 321 us (now 303), a step
-//                      under FP8 Q K^T 326 us (now 289), a 1080P step 6.22 ms (now 5.57).  96 + 32:
-//                      P V of the first part (384 cycles) covers the second's arithmetic (~190).
+//                      both took 1230; a denoising step at 480P then ran 321 us (303 in two parts,
+//                      298 with the shorter waits since), a step under FP8 Q K^T 326 us (289; 276), a
+//                      1080P step 6.22 ms (5.57; 5.51).  96 + 32: P V of the first part (384 cycles)
+//                      covers the second's arithmetic (~190).
 // TMEM columns: S0 0-127, S1 128-255, O0 256.., O1 256+D.. (512 allocated).
 // FP8_QK variant (D = 128): the K tiles hold E4M3 codes (one 128-byte swizzle atom per row,
 // from the view arena's E4M3 copy); the bf16 Q tiles are loaded as usual and each softmax
@@ -503,7 +504,7 @@ __device__ __forceinline__ void merge_rows(uint32_t part, uint32_t ml, int S, in
 // merge: both warpgroups own the same rows, warpgroup t over key tiles t, t + 2, .. (the two sets of S,
 // P and O in tensor memory are the key sets' instead of the query tiles'), merged at the end like two
 // more splits.  Per key tile a CTA takes 0.65 of the time for twice the K and V per query (when it pays:
-// choose_attention_plan).  6 heads, 808 queries, 2828 and 2020 keys, D = 128: 17.2 -> 14.4 us a launch.
+// choose_attention_plan).  6 heads, 808 queries, 2828 and 2020 keys, D = 128: 16.8 -> 14.3 us a launch.
 template <int D, bool kSplit, bool kFp8, bool kFp8PV = false, bool kOne = false>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -1059,12 +1060,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 // CTAs handles one (head, 128-row query tile), each CTA a k-th of the key tiles (two fill the SMs
 // in about three even waves at 480P instead of two, the second half empty; small windows take
 // more, see launch_head_profile); the other CTAs write their row statistics into the first's shared
-// memory (distributed shared memory, one cluster barrier), and the first merges the ranges.
+// memory (distributed shared memory, between two cluster barriers), and the first merges the ranges.
 // What bounds it: the statistics warps (the exponentials of a tile alone hold an SM sub-partition's
 // special-function unit for 512 cycles, as long as the MMAs take; each is active 63% of the time).
 // With one set of statistics warps per CTA the two CTAs of an SM fell into step, computing and
-// waiting at the same time.  12 heads, 4680 queries, 34320 keys: 372 us (405 with one set, its loads
-// not overlapped and a branch per key in tiles of two classes; D = 64 320, was 389); 8 heads, 534
+// waiting at the same time.  12 heads, 4680 queries, 34320 keys, launches back to back: 372 us (405 with one
+// set, its loads not overlapped and a branch per key in tiles of two classes; D = 64 320, was 389), 351-402 by
+// box for a launch on a flushed L2; 8 heads, 534
 // queries, 1246 keys, D = 64: 10.4 us (16.4 with two CTAs per query tile).  Tried: S released before
 // the sums (registers for 128 columns), no faster; loads running ahead into the next tile, slower; the
 // query tile in tensor memory, which halves the operand fetch from shared memory (8 KB in the 64

@@ -104,13 +104,16 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // (set-up, first loads, epilogue, and with k > 1 the merge), on the `clusters[k]` clusters that the
 // device holds at once.  Grids that leave SMs idle (few heads or queries) or whose last wave is short
 // are where splits pay; CTAs of one query tile take 0.65 of the time per key tile, so less per CTA but more
-// per query, and merge half the bytes: they pay on small grids.  Measured, us (query tiles per CTA, k), two query
-// tiles and no split / best with two / best with one: 6 heads, 808 queries, 2828 and 2020 keys 33.4 / 17.2
-// (2, 5) / 14.4 (1, 3); 1 head, 328 queries, 2132 keys 26.0 / 13.7 (2, 6) / 10.1 (1, 6); 2 heads, 4680
-// queries, 13000 and 7800 keys 126 / 51.5 (2, 3) / 43.5 (1, 2); 4 heads, 2412 queries, 13132 and 4020 keys
-// 128 / 42.2 (2, 4) / 44.1 (1, 2); 12 heads, 4680 queries, 15600 keys 314 / 280 (2, 2) / 316 (1, 1), 25480
-// and 7800 keys 286 (2, 1) / 286 / 333 (1, 1).  The overheads are fitted to such sweeps: over 16 shapes the choice
-// was the fastest measured in 14 and within 3% and 6% of it in two.
+// per query, and merge half the bytes: they pay on small grids.  Measured back to back, us (query tiles per CTA,
+// k), two query tiles and no split / best with two / best with one, bf16 and then FP8: 6 heads, 808 queries, 2828
+// and 2020 keys 33.7 / 16.8 (2, 5) / 14.3 (1, 3), 31.9 / 16.8 / 14.3; 1 head, 328 queries, 2132 keys 26.4 / 14.1
+// (2, 6) / 10.4 (1, 6), 25.1 / 13.9 / 10.3; 2 heads, 4680 queries, 14820 and 7800 keys 144 / 56.4 (2, 3) / 47.7
+// (1, 2), 127 / 51.9 / 39.7; 4 heads, 2412 queries, 13132 and 4020 keys 129 / 42.2 (2, 4) / 44.0 (1, 2), 117 /
+// 40.7 / 40.8; 12 heads, 4680 queries, 15600 and 10920 keys 311 / 259 (2, 2) / 307 (1, 1), 277 / 235 / 239, 25480
+// and 7800 keys 259 (2, 1) / 259 / 324 (1, 1), 227 / 227 / 261.  The constants are fitted to such sweeps in bf16 at
+// D = 128 and serve every precision: over 11 shapes in bf16, FP8_QK, FP8 and D = 64 the choice was within 1% of the
+// fastest of the 16 plans in 38 of 44, and at worst 4-8% from it (8 heads, 1494 queries, 8134 and 2490 keys: 33.4
+// for (2, 4) against 31.4 for (1, 2); FP8, 12 heads, 16380 and 7800 keys: 205 for (2, 2) against 196 for (1, 1)).
 struct AttnPlan {
   int one_qtile, kv_splits;
 };

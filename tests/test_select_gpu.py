@@ -1,5 +1,5 @@
 """Selection with many segments per frame (radix select): sizes around the thread count, budgets from
-none to all, ties, and every rule, against the oracle."""
+none to all, ties, and every rule, against the oracle; configurations at the limits of shared memory."""
 import os
 import subprocess
 import sys
