@@ -872,12 +872,12 @@ def run_stack(local_rank, attn_precision="bf16"):
 # removed) the capture was taken on: a figure is reported only while that code is unchanged.
 NCU_TRAFFIC = {
     "480p_layer": {
-        "attend": ("fk_attn.cu", "56d9abeaf551", 119190000),
-        "attend_fp8": ("fk_attn.cu", "56d9abeaf551", 92200000),
-        "attend_fp8pv": ("fk_attn.cu", "56d9abeaf551", 65810000),
+        "attend": ("fk_attn.cu", "90b07b56a988", 118980000),
+        "attend_fp8": ("fk_attn.cu", "90b07b56a988", 92110000),
+        "attend_fp8pv": ("fk_attn.cu", "90b07b56a988", 65890000),
         "append": ("fk_copy.cu", "e3a1045fec8c", 54790000),
         "compact": ("fk_copy.cu", "e3a1045fec8c", 58560000),
-        "score": ("fk_score.cu", "438a4f62fc08", 35970000),
+        "score": ("fk_score.cu", "1bc903628fd4", 35970000),
     },
 }
 

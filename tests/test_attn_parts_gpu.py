@@ -1,5 +1,6 @@
 """Attention: the running maximum raised in either part of a key tile (keys 0-95 and 96-127 are
-handed to the tensor cores separately), in the first, a middle and the ragged last tile."""
+handed to the tensor cores separately), in the first, a middle and the ragged last tile; every launch
+plan (query tiles per CTA, key splits) by itself."""
 import numpy as np
 import pytest
 
